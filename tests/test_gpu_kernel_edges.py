@@ -1,0 +1,37 @@
+"""Kernel variants at the sizes where a tile, a remainder or a route changes, against the CPU FP64
+oracle (tolerances of the parity tests: 1e-10 of peak in FP64, 1e-5 in FP32)."""
+import numpy as np
+import pytest
+
+import synthetic as syn
+from oracle import core, noise
+from _helpers import TOL, qgrid_tuple, rel_err_of_peak, to_library
+
+pytestmark = pytest.mark.gpu
+PREC = [(0, "fp64"), (1, "fp32")]
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    import paper_1809_07088_gb300 as ds
+    c = ds.Context(0)
+    yield c
+    c.close()
+
+
+@pytest.mark.parametrize("prec,tag", PREC)
+@pytest.mark.parametrize("m_,mp", [(2, 2), (3, 3), (2, 5), (4, 8)])
+def test_lanczos_point_weights_near_bragg_and_half_positions(ctx, prec, tag, m_, mp):
+    """Points on, and 1e-12 to 1e-6 beside, Bragg positions and the half positions between them, where
+    the weights switch between the limit, the nearest and the next Bragg position; tap counts of every
+    register size (4, 10, 32), equal and different sine arguments."""
+    m = syn.small_case(syn.OCC, cells=(6, 5, 4), nsite=2, nmodels=1, seed=231)
+    lm = to_library(ctx, m)
+    d = np.array([0.0, 1e-12, -1e-12, 3e-9, -3e-8, 1e-6, -1e-6, 0.5, 0.5 + 1e-9, 0.5 - 1e-9, 0.25])
+    Q = np.stack(np.meshgrid(d + 2.0, d[::-1] - 3.0, d[::3], indexing="ij"), -1).reshape(-1, 3)
+    hkl = Q / np.array(m.cells, dtype=np.float64)
+    got, _ = lm.intensity_points(hkl, disorder=0, mode=1, precision=prec, lanczos_m=m_, lanczos_mprime=mp)
+    sel = np.arange(0, Q.shape[0], 7)
+    want = noise.lanczos_resample(lambda G: core.occupancy_intensity_fft(m, G, 1),
+                                  (hkl * np.array(m.cells))[sel], m_, mp)
+    assert rel_err_of_peak(got[sel], want) < TOL[tag]
