@@ -1092,7 +1092,7 @@ ds_status plan_and_run(ds_model *M, const ds_qgrid *q, const ds_opts *o, T *d_ou
         T *dw = (T *)ws.get(sizeof(T) * (size_t)nsite * ecnt[0] * ecnt[1] * ecnt[2]);
         if (ws.failed) return ds_fail(ctx, DS_ERR_OOM, "device allocation failed (Debye-Waller factors)");
         ProfScope ps(ctx, "debye_waller", st);
-        debye_waller_grid<T>(M, eg0, ecnt, dw, st);
+        debye_waller_grid<T>(M, eg0, ecnt, dw, ws, st);
         p.dw = dw;
         p.force_plain = 1;
     }

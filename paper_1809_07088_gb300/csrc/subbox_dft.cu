@@ -459,7 +459,207 @@ template <typename T> struct DwParams {
     long long npts;
     long long site_stride, pt_stride;
     T *out;
+    const double *xc;       // grid: max |Q.u| at the 8 corners of the grid
+    int *route;             // grid: (P, taylor, wide), written by k_dw_moments (null: direct sum only)
+    double gscale[3];       // grid: largest |g_a| (r.l.u.)
+    double xstep[3];        // grid: 1 / (n_a gs_a): x_a = G_a xstep_a
+    int nchunk;             // grid: sample chunks of the moment sums
+    double *part, *mom;     // grid: moments [chunk][site][DW_T] and [site][DW_T]
 };
+
+// ---- T_mu(G) on a grid from the moments of the displacements -----------------------------------
+// The even part of Eq. dw is a polynomial in g up to the remainder bound of Section III C:
+//     T_mu(G) = sum_{n even <= P} (-1)^(n/2) sum_{a+b+c=n} x1^a x2^b x3^c <v1^a v2^b v3^c> / (a! b! c!),
+// v_j = gs_j b*_j.u, x_j = g_j / gs_j (|x_j| <= 1), P the smallest order with x_max^(P+1)/(P+1)! below
+// the working precision.  The moments are sums over the lattice points (once per site, not once per
+// voxel), the polynomial is evaluated axis by axis (P + 1 multiply-adds per voxel), in place of one
+// complex rotation per voxel and lattice point.  x_max stays on the device: k_dw_moments derives
+// the route from it for the kernels that follow, so the request needs no read-back; the direct kernel
+// returns at once when the moments serve.  Sums are taken in FP64 (partial sums of 16 terms in the working type); the
+// polynomial in the working type while x_max <= 2 (cosh x_max bounds the cancellation), else in FP64.
+// 16 sites, 20^3 cells, 81^3 voxels, x_max about 0.5: the request takes 0.25 ms, 17.4 ms by the direct
+// sum (whose FP32 rotations left 1.6e-5 of the result; 1.1e-7 by the moments).  A grid of fewer voxels
+// than monomials keeps the direct sum: one rotation per voxel and point costs about a monomial's product.
+constexpr int DW_PCAP = 28;
+constexpr int DW_T = (DW_PCAP + 1) * (DW_PCAP + 2) * (DW_PCAP + 3) / 6;
+constexpr int DW_SUB = 64;   // samples staged per pass
+struct DwRoute {
+    int P, taylor, wide;     // wide: evaluate in FP64
+};
+// remainder allowed: a quarter of an FP32 ulp of 1, or below FP64 rounding
+template <typename T> __device__ __forceinline__ constexpr double dw_eps() { return sizeof(T) == 4 ? 1.5e-8 : 1e-17; }
+__device__ __forceinline__ DwRoute dw_route(const double *xc, double eps, long long nvox) {
+    double x = 0.0;
+    for (int c = 0; c < 8; ++c) x = fmax(x, xc[c]);
+    DwRoute r;
+    double term = x;   // x^(P+1) / (P+1)!
+    int P = 0;
+    while (P <= DW_PCAP && !(term <= eps)) {
+        ++P;
+        term *= x / (P + 1);
+    }
+    P = max(P & ~1, 2);   // odd orders do not enter; P >= 2 lets a non-finite displacement reach the sums
+    const long long T2 = (long long)(P + 1) * (P + 2) * (P + 3) / 6;
+    r.P = P;
+    // moments cost T2 / 2 products per lattice point, the direct sum one rotation per voxel and point
+    r.taylor = P <= DW_PCAP && T2 <= nvox;
+    r.wide = eps < 1e-12 || x > 2.0;
+    return r;
+}
+// index of monomial (a, b, 0) in the lexicographic list of order P
+__device__ __forceinline__ int dw_t0(int P, int a, int b) {
+    const int P1 = P + 1, q = P1 - a;
+    return (P1 * (P1 + 1) * (P1 + 2) - q * (q + 1) * (q + 2)) / 6 + b * (P - a + 1) - b * (b - 1) / 2;
+}
+
+// part[chunk][site][t]: sums of v1^a v2^b v3^c / (a! b! c!) over the chunk's samples (even orders)
+template <typename T>
+__global__ void __launch_bounds__(256) k_dw_moments(const __grid_constant__ DwParams<T> p) {
+    __shared__ DwRoute rt;
+    if (threadIdx.x == 0) {
+        rt = dw_route(p.xc, dw_eps<T>(), p.npts);
+        if (blockIdx.x == 0 && blockIdx.y == 0) p.route[0] = rt.P, p.route[1] = rt.taylor, p.route[2] = rt.wide;
+    }
+    __syncthreads();
+    if (!rt.taylor) return;
+    const int P = rt.P, P1 = P + 1, s = blockIdx.y, ch = blockIdx.x;
+    constexpr int RS = DW_SUB + 1;                 // rows one apart in the banks
+    extern __shared__ __align__(16) unsigned char dw_raw[];
+    T *pw = (T *)dw_raw;                            // [axis][e][sample]
+    __shared__ T inv_e[DW_PCAP + 1];                // 1 / (e + 1)
+    if (threadIdx.x <= DW_PCAP) inv_e[threadIdx.x] = (T)(1.0 / (threadIdx.x + 1));
+    const long long nsamp = (long long)p.nmodels * p.ncell;
+    const long long per = (nsamp + p.nchunk - 1) / p.nchunk;
+    const long long j_lo = ch * per, j_hi = min(nsamp, j_lo + per);
+    double *dst = p.part + ((size_t)ch * p.nsite + s) * DW_T;
+    // the thread's (a, b) chains: all c of one parity
+    const int nab = P1 * (P1 + 1) / 2;
+    for (int base = 0; base < nab * P1; base += 256 * 8) {
+        // up to eight monomials per thread and sweep of the samples
+        int ia[8], ib[8], ic[8];
+        double acc[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int it = base + u * 256 + threadIdx.x;
+            acc[u] = 0.0;
+            ia[u] = -1;
+            ib[u] = ic[u] = 0;
+            if (it < nab * P1) {
+                const int ab = it / P1, c = it - ab * P1;
+                int a = 0, off = ab;
+                while (off >= P1 - a) off -= P1 - a, ++a;
+                if (a + off + c <= P && ((a + off + c) & 1) == 0) ia[u] = a, ib[u] = off, ic[u] = c;
+            }
+        }
+        for (long long j0 = j_lo; j0 < j_hi; j0 += DW_SUB) {
+            const int n = (int)min((long long)DW_SUB, j_hi - j0);
+            __syncthreads();
+            for (int i = threadIdx.x; i < 3 * DW_SUB; i += 256) {
+                const int ax = i / DW_SUB, k = i - ax * DW_SUB;
+                double v = 0.0;
+                if (k < n) {
+                    const long long j = j0 + k, m = j / p.ncell, cell = j - m * p.ncell;
+                    const size_t at = 3 * (((size_t)m * p.nsite + s) * p.ncell + cell);
+                    v = p.gscale[ax] * (p.recip[3 * ax] * p.disp[at] + p.recip[3 * ax + 1] * p.disp[at + 1] +
+                                        p.recip[3 * ax + 2] * p.disp[at + 2]);
+                }
+                T q = k < n ? T(1) : T(0);
+                const T vt = (T)v;
+                for (int e = 0; e < P1; ++e) {
+                    pw[(ax * P1 + e) * RS + k] = q;
+                    q *= vt * inv_e[e];
+                }
+            }
+            __syncthreads();
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                if (ia[u] < 0) continue;
+                const T *x = pw + ia[u] * RS, *y = pw + (P1 + ib[u]) * RS, *z = pw + (2 * P1 + ic[u]) * RS;
+                for (int k0 = 0; k0 < DW_SUB; k0 += 16) {
+                    T t = T(0);
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) t = fma(x[k0 + k] * y[k0 + k], z[k0 + k], t);
+                    acc[u] += (double)t;
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (ia[u] >= 0) dst[dw_t0(P, ia[u], ib[u]) + ic[u]] = acc[u];
+    }
+}
+
+// mom[site][t] = (-1)^(n/2) mean of the monomial (chunks added in order; odd orders 0)
+template <typename T>
+__global__ void k_dw_reduce(const __grid_constant__ DwParams<T> p) {
+    if (!p.route[1]) return;
+    const int P = p.route[0], P1 = P + 1, s = blockIdx.y;
+    const double inv = 1.0 / ((double)p.nmodels * p.ncell);
+    for (int it = blockIdx.x * blockDim.x + threadIdx.x; it < P1 * P1 * P1; it += gridDim.x * blockDim.x) {
+        const int a = it / (P1 * P1), b = (it / P1) % P1, c = it % P1, n = a + b + c;
+        if (n > P) continue;
+        const int t = dw_t0(P, a, b) + c;
+        double v = 0.0;
+        if ((n & 1) == 0) {
+            for (int ch = 0; ch < p.nchunk; ++ch) v += p.part[((size_t)ch * p.nsite + s) * DW_T + t];
+            v *= (n & 2) ? -inv : inv;
+        }
+        p.mom[(size_t)s * DW_T + t] = v;
+    }
+}
+
+// CTA: one site and one G1; N[b][c] = sum_a x1^a mom, then per tile of DW_ROWS rows G2
+// L[row][c] = sum_b x2^b N[b][c], then the voxels of the rows by Horner in x3
+constexpr int DW_ROWS = 32, DW_ETHR = 128;
+template <typename T, typename CT>
+__device__ __forceinline__ void dw_eval_body(const DwParams<T> &p, int P, CT *N, CT *L) {
+    const int P1 = P + 1, s = blockIdx.y, i0 = blockIdx.x, tid = threadIdx.x;
+    auto xat = [&](int a, int i) { return (CT)((double)(p.g0[a] + i) * p.xstep[a]); };
+    const double *mom = p.mom + (size_t)s * DW_T;
+    const CT x1 = xat(0, i0);
+    for (int it = tid; it < P1 * P1; it += DW_ETHR) {
+        const int b = it / P1, c = it - b * P1;
+        if (b + c > P) continue;
+        CT v = CT(0);
+        for (int a = P - b - c; a >= 0; --a) v = fma(v, x1, (CT)mom[dw_t0(P, a, b) + c]);
+        N[b * P1 + c] = v;
+    }
+    const int c1 = p.cnt[1], c2 = p.cnt[2];
+    T *out = p.out + (size_t)s * p.site_stride + (size_t)i0 * c1 * c2;
+    for (int r0 = 0; r0 < c1; r0 += DW_ROWS) {
+        const int nr = min(DW_ROWS, c1 - r0);
+        __syncthreads();
+        for (int it = tid; it < nr * P1; it += DW_ETHR) {
+            const int r = it / P1, c = it - r * P1;
+            const CT x2 = xat(1, r0 + r);
+            CT v = CT(0);
+            for (int b = P - c; b >= 0; --b) v = fma(v, x2, N[b * P1 + c]);
+            L[r * P1 + c] = v;
+        }
+        __syncthreads();
+        for (int it = tid; it < nr * c2; it += DW_ETHR) {
+            const int r = it / c2, i2 = it - r * c2;
+            const CT x3 = xat(2, i2);
+            const CT *l = L + r * P1;
+            CT v = l[P];
+            for (int c = P - 1; c >= 0; --c) v = fma(v, x3, l[c]);
+            out[(size_t)(r0 + r) * c2 + i2] = (T)v;
+        }
+    }
+}
+template <typename T>
+__global__ void __launch_bounds__(DW_ETHR) k_dw_eval(const __grid_constant__ DwParams<T> p) {
+    if (!p.route[1]) return;
+    extern __shared__ __align__(16) unsigned char dw_raw[];
+    const int P = p.route[0], P1 = P + 1;
+    if (sizeof(T) == 8 || p.route[2]) {
+        double *N = (double *)dw_raw;
+        dw_eval_body<T, double>(p, P, N, N + P1 * P1);
+    } else {
+        T *N = (T *)dw_raw;
+        dw_eval_body<T, T>(p, P, N, N + P1 * P1);
+    }
+}
 
 template <typename T>
 __global__ void __launch_bounds__(DW_THREADS) k_debye_waller(const __grid_constant__ DwParams<T> p) {
@@ -506,11 +706,13 @@ __global__ void __launch_bounds__(DW_THREADS) k_debye_waller(const __grid_consta
 // sincos), then walks the row by z <- z w (four multiply-adds per voxel, no SFU operation).
 template <typename T, int VPT>
 __global__ void __launch_bounds__(DW_THREADS) k_debye_waller_rows(const __grid_constant__ DwParams<T> p) {
+    if (p.route && p.route[1]) return;   // k_dw_eval writes the factors
     __shared__ float4 stage[DW_STAGE];
     const int s = blockIdx.y;
     const int nseg = (p.cnt[2] + VPT - 1) / VPT;
     const long long nwork = (long long)p.cnt[0] * p.cnt[1] * nseg;
-    const long long wi = (long long)blockIdx.x * DW_THREADS + threadIdx.x;
+    for (long long w0 = (long long)blockIdx.x * DW_THREADS; w0 < nwork; w0 += (long long)gridDim.x * DW_THREADS) {
+    const long long wi = w0 + threadIdx.x;
     const bool live = wi < nwork;
     const long long ww = live ? wi : nwork - 1;
     const long long row = ww / nseg;
@@ -557,12 +759,12 @@ __global__ void __launch_bounds__(DW_THREADS) k_debye_waller_rows(const __grid_c
             }
         }
     }
-    if (!live) return;
     const T inv = T(1) / (T)nsamp;
     const size_t v0 = ((size_t)i0 * p.cnt[1] + i1) * p.cnt[2] + i2_0;
 #pragma unroll
     for (int j = 0; j < VPT; ++j)
-        if (i2_0 + j < p.cnt[2]) p.out[(size_t)s * p.site_stride + v0 + j] = acc[j] * inv;
+        if (live && i2_0 + j < p.cnt[2]) p.out[(size_t)s * p.site_stride + v0 + j] = acc[j] * inv;
+    }
 }
 
 template <typename T> DwParams<T> dw_params(const ds_model *M, bool weights) {
@@ -716,24 +918,54 @@ ds_status run_debye_waller(ds_model *Mdl, const double *hkl, long long npts, int
 }  // namespace
 
 // T_mu(G) on the computing grid of a magnetic request, [site][voxel] (api.cu)
-template <typename T> void debye_waller_grid(const ds_model *M, const int g0[3], const int cnt[3], T *out, cudaStream_t st) {
+template <typename T>
+void debye_waller_grid(const ds_model *M, const int g0[3], const int cnt[3], T *out, Scratch &ws, cudaStream_t st) {
     DwParams<T> d = dw_params<T>(M, false);
     for (int a = 0; a < 3; ++a) {
         d.g0[a] = g0[a];
         d.cnt[a] = cnt[a];
+        double gs = std::max(fabs((double)g0[a]), fabs((double)g0[a] + cnt[a] - 1)) / M->n[a];
+        if (!(gs > 0)) gs = 1.0;
+        d.gscale[a] = gs;
+        d.xstep[a] = 1.0 / (M->n[a] * gs);
     }
     d.npts = (long long)cnt[0] * cnt[1] * cnt[2];
     d.site_stride = d.npts;
     d.pt_stride = 1;
     d.out = out;
+    const long long nsamp = (long long)d.nmodels * d.ncell;
+    // moment route: chunks of at least 256 lattice points, about two CTAs per SM over the sites
+    d.nchunk = (int)std::max<long long>(1, std::min<long long>((nsamp + 255) / 256, (152 * 2 + d.nsite - 1) / d.nsite));
+    double *xc = (double *)ws.get(sizeof(double) * 9);
+    double *mom = (double *)ws.get(sizeof(double) * DW_T * d.nsite);
+    double *part = (double *)ws.get(sizeof(double) * DW_T * d.nsite * (size_t)d.nchunk);
+    int *route = (int *)ws.get(sizeof(int) * 3);
+    if (!ws.failed) {
+        d.route = route;
+        Corners corners;
+        box_corners(M, g0, cnt, corners.v);
+        corner_xmax((int)(nsamp * d.nsite), M->d_disp, corners, xc, st);
+        d.xc = xc;
+        d.mom = mom;
+        d.part = part;
+        const size_t sm = sizeof(T) * 3 * (DW_PCAP + 1) * (DW_SUB + 1);
+        if (sm > 48 * 1024) cudaFuncSetAttribute(k_dw_moments<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        k_dw_moments<T><<<dim3((unsigned)d.nchunk, (unsigned)d.nsite), 256, sm, st>>>(d);
+        k_dw_reduce<T><<<dim3(8, (unsigned)d.nsite), 256, 0, st>>>(d);
+        const size_t se = sizeof(double) * (DW_PCAP + 1) * (DW_PCAP + 1 + DW_ROWS);
+        k_dw_eval<T><<<dim3((unsigned)cnt[0], (unsigned)d.nsite), DW_ETHR, se, st>>>(d);
+        count_launches(3);
+    } else {
+        ws.failed = false;   // no scratch for the moments: the direct sum needs none
+    }
     constexpr int VPT = 8;
     const long long nwork = (long long)cnt[0] * cnt[1] * ((cnt[2] + VPT - 1) / VPT);
-    const dim3 grid((unsigned)((nwork + DW_THREADS - 1) / DW_THREADS), (unsigned)d.nsite);
-    k_debye_waller_rows<T, VPT><<<grid, DW_THREADS, 0, st>>>(d);
+    const long long nb = std::min<long long>((nwork + DW_THREADS - 1) / DW_THREADS, std::max(1, 152 * 64 / d.nsite));
+    k_debye_waller_rows<T, VPT><<<dim3((unsigned)nb, (unsigned)d.nsite), DW_THREADS, 0, st>>>(d);
     count_launches(1);
 }
-template void debye_waller_grid<float>(const ds_model *, const int *, const int *, float *, cudaStream_t);
-template void debye_waller_grid<double>(const ds_model *, const int *, const int *, double *, cudaStream_t);
+template void debye_waller_grid<float>(const ds_model *, const int *, const int *, float *, Scratch &, cudaStream_t);
+template void debye_waller_grid<double>(const ds_model *, const int *, const int *, double *, Scratch &, cudaStream_t);
 
 extern "C" ds_status ds_request_subbox_points(ds_model *Mdl, const int32_t *origins, int64_t norigin, const double *hkl,
                                               int64_t npts, int hkl_is_device, const ds_opts *o, void *out,

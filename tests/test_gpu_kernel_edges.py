@@ -35,3 +35,22 @@ def test_lanczos_point_weights_near_bragg_and_half_positions(ctx, prec, tag, m_,
     want = noise.lanczos_resample(lambda G: core.occupancy_intensity_fft(m, G, 1),
                                   (hkl * np.array(m.cells))[sel], m_, mp)
     assert rel_err_of_peak(got[sel], want) < TOL[tag]
+
+
+@pytest.mark.parametrize("prec,tag", PREC)
+@pytest.mark.parametrize("sigma", [0.0, 0.02, 0.2, 0.45, 3.0])
+@pytest.mark.parametrize("count", [(1, 1, 1), (5, 37, 3), (9, 11, 13)])
+def test_debye_waller_grid_routes(ctx, prec, tag, sigma, count):
+    """T_mu(G) on grids by the moments of the displacements (polynomial in the working type, in FP64)
+    and by the direct sum, chosen on the device from x_max and the voxel count: no displacement, small
+    and large ones, one voxel, more rows than a tile, a grid away from the origin."""
+    m = syn.small_case(syn.SPIN, cells=(6, 5, 4), nsite=3, nmodels=3, seed=232)
+    rng = np.random.default_rng(5)
+    m.disp = (sigma * rng.standard_normal(m.spins.shape)).astype(np.float32)
+    g0 = (-3, 2, -1)
+    m.qgrid = syn.QGrid(h0=tuple(g / n for g, n in zip(g0, m.cells)), step=tuple(1.0 / n for n in m.cells), count=count)
+    lm = to_library(ctx, m)
+    got, _ = lm.intensity(qgrid_tuple(m.qgrid), disorder=1, mode=0, precision=prec, dw_coupling=1)
+    want = core.magnetic_intensity_fft(m, m.qgrid.g_index(m.cells), 0, dw=True)
+    scale = np.max(core.magnetic_intensity_fft(m, m.qgrid.g_index(m.cells), 0))
+    assert np.max(np.abs(got.reshape(-1) - want)) / scale < TOL[tag]
