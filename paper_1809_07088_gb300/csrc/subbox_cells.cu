@@ -1,0 +1,587 @@
+// Sub-box sums at arbitrary wavevectors from cell amplitudes shared by the boxes (Section V A; the same
+// sum as subbox_dft.cu, regrouped).
+//
+// With many origins a lattice point lies in several boxes: norigin n_sb^3 / (nmodels n1 n2 n3) of them
+// on average.  The amplitude of a cell,
+//     A_R(Q) = sum_mu phi_mu(Q) a_{R,mu}(Q),   a = delta, M or delta exp(i Q.u),
+// carries no box, so it is formed once per cell and point instead of once per box; a box then costs
+//     F_o = sum_d1 e1^d1 sum_d2 e2^d2 L_{o + (d1, d2, 0)},   L_R = sum_d3 e3^d3 A_{R + (0, 0, d3)},
+// e_a = exp(2 pi i h_a), with cells wrapped and phases not (open boxes).  The line sums L are formed as
+// the cells of a row are walked (the last eight amplitudes stay in registers), so a box reads n_sb^2
+// values per point.  For displacements the bound moves from one SFU (sin, cos) pair per atom and box to
+// one per atom, plus the L2 traffic of the line sums.
+//
+// Points are taken in chunks whose line sums stay in the L2 (SX_L2 bytes), one point per thread: the
+// loads and stores of a warp are 32 consecutive points.  Per chunk: line sums (grid: points x rows of
+// cells), the Debye-Waller means from the same exponentials (DIFFUSE displacements), the boxes (grid:
+// points x origin chunks).  Partial sums are added in a fixed order.
+//
+// fcc 32^3 (131,072 atoms), 2516 origins, n_sb = 5, 40,401 points, FP32: 9.8 ms (29.5 ms box by box, at
+// 0.75 of the SFU rate); per chunk of 256 points the line sums take about 34 us (instruction issue 71 %),
+// the means 4, the boxes 22.
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+#include <type_traits>
+
+#include "api_internal.h"
+#include "subbox_points.h"
+
+using namespace ds;
+
+namespace {
+
+constexpr int SX_T = 128;                     // points per block
+constexpr size_t SX_L2 = 64u << 20;           // line sums of a chunk
+constexpr size_t SX_MOST = 1024u << 20;       // and at most, for one block of points over large ensembles
+constexpr long long SX_PREP = 65536;          // points whose constants are held at once
+constexpr int SX_RING = 8;                    // amplitudes of a row kept in registers
+
+template <typename T> struct SxParams {
+    int nsite, nsb, n1, n2, n3, ncell, nmodels, diffuse;
+    const SbSite *site;
+    const uint8_t *occ;
+    const float *vec;
+    const double *mean;
+    const double *hkl;
+    long long npts;                 // points of the request
+    long long p0, np;               // points whose constants are held: [p0, p0 + np)
+    long long q0;                   // first of them in this chunk, relative to p0
+    int nq, ld;                     // points of the chunk, and padded to whole blocks
+    long long ldp;                  // stride of the constants
+    double recip[9];
+    c_t<T> *phi;                    // [site][ldp]: phi_mu; displacements (b f, Q.r_mu in cycles)
+    c_t<T> *e;                      // [axis][ldp]
+    T *Q;                           // [axis][ldp]: Q / 2 pi (cycles per A) for displacements, Q for moments
+    c_t<T> *B, *K;                  // displacements: box sum of exp(2 pi i Q.d); others: mean amplitude [comp][ldp]
+    c_t<T> *A, *L;                  // [comp][model cell][ld]; A: amplitudes where the line sums take their own pass
+    T *dwp, *dwm;                   // [row block][site][ld]: sums of w cos(Q.u); [site][ld]: their mean
+    int rows_per, nrb;              // rows of cells per block, row blocks
+    const int4 *origins;
+    long long norigin, per_chunk;
+    T *partial;                     // [origin chunk][npts]
+};
+
+// per-point constants (FP64, stored in the working type)
+template <typename T, int KIND> __global__ void __launch_bounds__(SX_T) k_sx_prep(const __grid_constant__ SxParams<T> p) {
+    const long long j = (long long)blockIdx.x * SX_T + threadIdx.x;
+    if (j >= p.ldp) return;
+    const long long q = p.p0 + min(j, p.np - 1);   // padding repeats the last point
+    const double h[3] = {p.hkl[3 * q], p.hkl[3 * q + 1], p.hkl[3 * q + 2]};
+    double Qd[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        Qd[a] = h[0] * p.recip[a] + h[1] * p.recip[3 + a] + h[2] * p.recip[6 + a];
+        p.Q[a * p.ldp + j] = (T)(KIND == SB_DISP ? Qd[a] / TWO_PI_D : Qd[a]);
+    }
+    const double s2 = (Qd[0] * Qd[0] + Qd[1] * Qd[1] + Qd[2] * Qd[2]) / (FOUR_PI_D * FOUR_PI_D);
+    constexpr int NC = KIND == SB_SPIN ? 3 : 1;
+    double Kr[NC], Ki[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) Kr[c] = Ki[c] = 0.0;
+    for (int s = 0; s < p.nsite; ++s) {
+        const SbSite &S = p.site[s];
+        const double f = S.b * form_factor<double>(S.kind, S.coef, s2);
+        const double t = frac_w(h[0] * S.r[0] + h[1] * S.r[1] + h[2] * S.r[2]);
+        if (KIND == SB_DISP) {
+            p.phi[s * p.ldp + j] = mk<T>((T)f, (T)t);
+            continue;
+        }
+        double sn, cs;
+        sincospi(2.0 * t, &sn, &cs);
+        p.phi[s * p.ldp + j] = mk<T>((T)(f * cs), (T)(f * sn));
+        if (p.diffuse) {
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                const double m = p.mean[KIND == SB_SPIN ? 3 * s + c : s];
+                Kr[c] += f * cs * m;
+                Ki[c] += f * sn * m;
+            }
+        }
+    }
+    if (KIND != SB_DISP)
+#pragma unroll
+        for (int c = 0; c < NC; ++c) p.K[c * p.ldp + j] = mk<T>((T)Kr[c], (T)Ki[c]);
+    double Br = 1.0, Bi = 0.0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        double sn, cs;
+        sincospi(2.0 * frac_w(h[a]), &sn, &cs);
+        p.e[a * p.ldp + j] = mk<T>((T)cs, (T)sn);
+        double xr = 1.0, xi = 0.0, sr = 0.0, si = 0.0;   // sum_d e^d
+        for (int d = 0; d < p.nsb; ++d) {
+            sr += xr;
+            si += xi;
+            const double t = xr * cs - xi * sn;
+            xi = xr * sn + xi * cs;
+            xr = t;
+        }
+        const double t = Br * sr - Bi * si;
+        Bi = Br * si + Bi * sr;
+        Br = t;
+    }
+    if (KIND == SB_DISP) p.B[j] = mk<T>((T)Br, (T)Bi);
+}
+
+// x e + a for complex x, e, a
+template <typename C> __device__ __forceinline__ C cmad(C x, C e, C a) {
+    C r;
+    r.x = fma(x.x, e.x, fma(-x.y, e.y, a.x));
+    r.y = fma(x.x, e.y, fma(x.y, e.x, a.y));
+    return r;
+}
+
+// Line sums (LINE) or plain amplitudes of whole rows of cells.  The row loop is unrolled by the ring
+// length, so the ring is indexed by constants.  Displacements: the site phase Q.r_mu is added to each
+// atom's phase, so an atom costs three multiply-adds, one reduction, one (sin, cos) pair and two
+// multiply-adds; the sums of its (cos, sin) per site give the Debye-Waller mean.  Sites beyond nsite
+// (MAXS > nsite) are atoms of weight zero.  WGT: occupancies weight the displaced atoms.
+template <typename T, int KIND, int MAXS, bool LINE, bool WGT>
+__global__ void __launch_bounds__(SX_T, sizeof(T) == 4 && MAXS <= 4 && KIND != SB_SPIN ? 8 : 4) k_sx_rows(const __grid_constant__ SxParams<T> p) {
+    using C = c_t<T>;
+    constexpr int NC = KIND == SB_SPIN ? 3 : 1;
+    extern __shared__ __align__(16) unsigned char sx_raw[];
+    const int nsite = p.nsite, nsb = p.nsb, n3 = p.n3, tid = threadIdx.x;
+    float4 *atoms = (float4 *)sx_raw;                        // [n3][MAXS]
+    C *first = (C *)(sx_raw + sizeof(float4) * n3 * MAXS) + tid;   // LINE: [i][comp][SX_T], a row's first amplitudes
+    const int ql = blockIdx.x * SX_T + tid;
+    const long long j = p.q0 + ql;                     // < ldp: chunks are whole blocks
+    C phi[MAXS], wsum[KIND == SB_DISP ? MAXS : 1];
+#pragma unroll
+    for (int s = 0; s < MAXS; ++s) {
+        phi[s] = s < nsite ? p.phi[s * p.ldp + j] : mk<T>(T(0), T(0));
+        if (KIND == SB_DISP) wsum[KIND == SB_DISP ? s : 0] = mk<T>(T(0), T(0));
+    }
+    const C e3 = p.e[2 * p.ldp + j];
+    T Qx = T(0), Qy = T(0), Qz = T(0);
+    C K[NC];
+    if (KIND == SB_DISP) {
+        Qx = p.Q[j], Qy = p.Q[p.ldp + j], Qz = p.Q[2 * p.ldp + j];
+    } else {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) K[c] = p.K[c * p.ldp + j];
+    }
+    const int nrow = p.nmodels * p.n1 * p.n2;
+    const int row_lo = blockIdx.y * p.rows_per, row_hi = min(nrow, row_lo + p.rows_per);
+    const size_t cstride = (size_t)p.nmodels * p.ncell * p.ld;
+    for (int row = row_lo; row < row_hi; ++row) {
+        const int m = row / (p.n1 * p.n2), rr = row - m * p.n1 * p.n2;
+        __syncthreads();
+        for (int i = tid; i < n3 * MAXS; i += SX_T) {
+            const int s = i / n3, r3 = i - s * n3;
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (s < nsite) {
+                const size_t at = ((size_t)m * nsite + s) * p.ncell + (size_t)rr * n3 + r3;
+                if (KIND == SB_OCC) v.x = (float)p.occ[at];
+                else v = make_float4(p.vec[3 * at], p.vec[3 * at + 1], p.vec[3 * at + 2], WGT ? (float)p.occ[at] : 1.f);
+            }
+            atoms[r3 * MAXS + s] = v;
+        }
+        __syncthreads();
+        C h[NC][SX_RING];
+        C *dst = (LINE ? p.L : p.A) + ((size_t)row * n3) * p.ld + ql;
+        const int npos = LINE ? n3 + nsb - 1 : n3;
+        // STEADY: every cell of the group is on the row and ends a box line
+        auto group = [&](int r0, auto steady) {
+            constexpr bool STEADY = decltype(steady)::value;
+            C *d0 = dst + (ptrdiff_t)(LINE ? r0 - nsb + 1 : r0) * p.ld;
+#pragma unroll
+            for (int u = 0; u < SX_RING; ++u) {
+                const int r = r0 + u;
+                if (!STEADY && r >= npos) break;
+                C a[NC];
+                if (STEADY || r < n3) {
+                    const float4 *at = atoms + r * MAXS;
+                    if (KIND == SB_DISP) {
+                        a[0] = mk<T>(T(0), T(0));
+#pragma unroll
+                        for (int s = 0; s < MAXS; ++s) {
+                            const float4 v = at[s];
+                            const T t = fma(Qx, (T)v.x, fma(Qy, (T)v.y, fma(Qz, (T)v.z, phi[s].y)));
+                            T cs, sn;
+                            sincos_cycles(frac_w(t), cs, sn);
+                            if (WGT) {
+                                cs *= (T)v.w;
+                                sn *= (T)v.w;
+                            }
+                            C &ws = wsum[KIND == SB_DISP ? s : 0];
+                            ws.x += cs;
+                            ws.y += sn;
+                            a[0].x = fma(phi[s].x, cs, a[0].x);
+                            a[0].y = fma(phi[s].x, sn, a[0].y);
+                        }
+                    } else {
+#pragma unroll
+                        for (int c = 0; c < NC; ++c) a[c] = mk<T>(-K[c].x, -K[c].y);
+#pragma unroll
+                        for (int s = 0; s < MAXS; ++s) {
+                            const float4 v = at[s];
+                            const T x[3] = {(T)v.x, (T)v.y, (T)v.z};
+#pragma unroll
+                            for (int c = 0; c < NC; ++c) {
+                                a[c].x = fma(phi[s].x, x[c], a[c].x);
+                                a[c].y = fma(phi[s].y, x[c], a[c].y);
+                            }
+                        }
+                    }
+                    if (LINE && !STEADY && r < nsb - 1)
+#pragma unroll
+                        for (int c = 0; c < NC; ++c) first[(r * NC + c) * SX_T] = a[c];
+                } else {
+                    // the row wraps: its first amplitudes again
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) a[c] = first[((r - n3) * NC + c) * SX_T];
+                }
+                if (LINE) {
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) h[c][u] = a[c];
+                }
+                if (!LINE || STEADY || r >= nsb - 1) {
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) {
+                        C l = a[c];
+                        if (LINE) {
+#pragma unroll
+                            for (int i = 1; i < SX_RING; ++i) {
+                                if (i >= nsb) break;
+                                l = cmad(l, e3, h[c][(u - i + SX_RING) % SX_RING]);
+                            }
+                        }
+                        d0[c * cstride + (ptrdiff_t)u * p.ld] = l;
+                    }
+                }
+            }
+        };
+        for (int r0 = 0; r0 < npos; r0 += SX_RING) {
+            if (r0 >= SX_RING && r0 + SX_RING <= n3) group(r0, std::true_type{});
+            else group(r0, std::false_type{});
+        }
+    }
+    if (KIND == SB_DISP && p.diffuse) {
+        // sum of w cos(Q.u) = Re[exp(-iQ.r_mu) sum of w exp(i(Q.u + Q.r_mu))]
+#pragma unroll
+        for (int s = 0; s < MAXS; ++s)
+            if (s < nsite) {
+                T cs, sn;
+                sincos_cycles(phi[s].y, cs, sn);
+                const C ws = wsum[KIND == SB_DISP ? s : 0];
+                p.dwp[((size_t)blockIdx.y * nsite + s) * p.ld + ql] = fma(ws.x, cs, ws.y * sn);
+            }
+    }
+}
+
+// line sums of boxes wider than the register ring, from the amplitudes
+template <typename T> __global__ void __launch_bounds__(SX_T) k_sx_line(const __grid_constant__ SxParams<T> p, int nc) {
+    using C = c_t<T>;
+    const int ql = blockIdx.x * SX_T + threadIdx.x;
+    const C e3 = p.e[2 * p.ldp + p.q0 + ql];
+    const size_t cells = (size_t)p.nmodels * p.ncell;
+    for (size_t i = blockIdx.y; i < cells * nc; i += gridDim.y) {
+        const size_t row = i / p.n3;
+        const int r3 = (int)(i - row * p.n3);
+        const C *a = p.A + row * p.n3 * p.ld + ql;
+        C l = mk<T>(T(0), T(0));
+        for (int d = p.nsb - 1; d >= 0; --d) {
+            int w = r3 + d;
+            if (w >= p.n3) w -= p.n3;
+            l = cmad(l, e3, a[(size_t)w * p.ld]);
+        }
+        p.L[i * p.ld + ql] = l;
+    }
+}
+
+// <w cos(Q.u)>_mu of the chunk's points: the row blocks' sums, by 32 threads per point in a fixed order
+constexpr int SX_MB = 32;
+template <typename T> __global__ void __launch_bounds__(32 * SX_MB) k_sx_mean(const __grid_constant__ SxParams<T> p) {
+    __shared__ T red[SX_MB][33];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, s = blockIdx.y;
+    const int ql = blockIdx.x * 32 + lane;
+    T t = T(0);
+#pragma unroll 16
+    for (int b = w; b < p.nrb; b += SX_MB) t += p.dwp[((size_t)b * p.nsite + s) * p.ld + ql];
+    red[w][lane] = t;
+    __syncthreads();
+    if (w == 0) {
+        T sum = T(0);
+#pragma unroll
+        for (int i = 0; i < SX_MB; ++i) sum += red[i][lane];
+        p.dwm[(size_t)s * p.ld + ql] = sum / (T)((double)p.nmodels * p.ncell);
+    }
+}
+
+// The boxes: sums over the line sums of a box's rows, eight loads in flight per thread; the element
+// offsets of each origin's wrapped rows are tabulated once per block.
+template <typename T, int KIND>
+__global__ void __launch_bounds__(SX_T) k_sx_boxes(const __grid_constant__ SxParams<T> p) {
+    using C = c_t<T>;
+    constexpr int NC = KIND == SB_SPIN ? 3 : 1;
+    constexpr int NB = SX_RING;
+    extern __shared__ __align__(16) unsigned char sx_raw[];
+    int *off1 = (int *)sx_raw;                      // [origin][nsb]: element offset of (model, o1 + d1, 0, o3)
+    int *off2 = off1 + p.per_chunk * p.nsb;         // [origin][nsb]: of row o2 + d2 within a plane
+    const int nsb = p.nsb;
+    const int ql = blockIdx.x * SX_T + threadIdx.x;
+    const long long j = p.q0 + ql;
+    const long long o0 = (long long)blockIdx.y * p.per_chunk;
+    const int no = (int)(min(p.norigin, o0 + p.per_chunk) - o0);
+    for (int i = threadIdx.x; i < no * nsb; i += SX_T) {
+        const int oi = i / nsb, d = i - oi * nsb;
+        const int4 og = p.origins[o0 + oi];
+        int w1 = og.y + d, w2 = og.z + d;   // o < n and d < n_sb <= n
+        if (w1 >= p.n1) w1 -= p.n1;
+        if (w2 >= p.n2) w2 -= p.n2;
+        off1[i] = ((og.x * p.n1 + w1) * p.n2 * p.n3 + og.w) * p.ld;
+        off2[i] = w2 * p.n3 * p.ld;
+    }
+    const C e1 = p.e[j], e2 = p.e[p.ldp + j];
+    C pw[NB];   // e2^u
+    pw[0] = mk<T>(T(1), T(0));
+#pragma unroll
+    for (int u = 1; u < NB; ++u) pw[u] = cmul(pw[u - 1], e2);
+    const C e2n = cmul(pw[NB - 1], e2);
+    C KB = mk<T>(T(0), T(0));
+    if (KIND == SB_DISP && p.diffuse) {
+        // K B, K = sum_mu phi_mu <w cos(Q.u)>_mu
+        C k = mk<T>(T(0), T(0));
+        for (int s = 0; s < p.nsite; ++s) {
+            const C ph = p.phi[s * p.ldp + j];
+            T cs, sn;
+            sincos_cycles(ph.y, cs, sn);
+            const T f = ph.x * p.dwm[(size_t)s * p.ld + ql];
+            k.x = fma(f, cs, k.x);
+            k.y = fma(f, sn, k.y);
+        }
+        KB = cmul(k, p.B[j]);
+    }
+    T Qv[3] = {T(0), T(0), T(0)};
+    if (KIND == SB_SPIN)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) Qv[a] = p.Q[a * p.ldp + j];
+    const size_t cstride = (size_t)p.nmodels * p.ncell * p.ld;
+    const C *L = p.L + ql;
+    __syncthreads();
+    T acc = T(0);
+    for (int oi = 0; oi < no; ++oi) {
+        C F[NC];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) F[c] = mk<T>(T(0), T(0));
+        for (int d1 = nsb - 1; d1 >= 0; --d1) {
+            const C *pl = L + off1[oi * nsb + d1];
+            C G[NC];
+#pragma unroll
+            for (int c = 0; c < NC; ++c) G[c] = mk<T>(T(0), T(0));
+            for (int t0 = (nsb - 1) / NB * NB; t0 >= 0; t0 -= NB) {
+                const int *o2 = off2 + oi * nsb + t0;
+                const int nt = nsb - t0;
+                C v[NB][NC];
+#pragma unroll
+                for (int u = 0; u < NB; ++u) {
+                    if (u >= nt) break;
+                    const C *at = pl + o2[u];
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) v[u][c] = at[c * cstride];
+                }
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    if (NB < nsb) G[c] = cmul(G[c], e2n);
+                    G[c] = cadd(G[c], v[0][c]);
+                }
+#pragma unroll
+                for (int u = 1; u < NB; ++u) {
+                    if (u >= nt) break;
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) cfma(G[c], pw[u], v[u][c]);
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < NC; ++c) F[c] = cmad(F[c], e1, G[c]);
+        }
+        T tot = T(0);
+        if (KIND == SB_DISP) F[0] = csub(F[0], KB);
+#pragma unroll
+        for (int c = 0; c < NC; ++c) tot += F[c].x * F[c].x + F[c].y * F[c].y;
+        if (KIND == SB_SPIN) {
+            const T q2 = Qv[0] * Qv[0] + Qv[1] * Qv[1] + Qv[2] * Qv[2];
+            if (q2 > T(0)) {
+                const T pr = Qv[0] * F[0].x + Qv[1] * F[1].x + Qv[2] * F[2].x;
+                const T pi = Qv[0] * F[0].y + Qv[1] * F[1].y + Qv[2] * F[2].y;
+                tot -= (pr * pr + pi * pi) / q2;
+            } else {
+                tot *= T(2) / T(3);
+            }
+        }
+        acc += tot;
+    }
+    if (ql < p.nq) p.partial[(size_t)blockIdx.y * p.npts + p.p0 + j] = acc;
+}
+
+template <typename T>
+__global__ void k_sx_sum(const T *__restrict__ partial, long long npts, int nchunk, double norm, T *__restrict__ out) {
+    for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < npts; q += (long long)gridDim.x * blockDim.x) {
+        double s = 0.0;
+        for (int c = 0; c < nchunk; ++c) s += (double)partial[(size_t)c * npts + q];
+        out[q] = (T)(s * norm);
+    }
+}
+
+template <typename T, int KIND, bool LINE, bool WGT> void launch_rows(const SxParams<T> &p, const dim3 &grid, cudaStream_t st) {
+    auto go = [&](auto kern, int maxs) {
+        // atoms of a row (<= 32 KB: n3 <= 128, nsite <= 16) and, for line sums, its first amplitudes
+        const size_t sm = sizeof(float4) * p.n3 * maxs +
+                          (LINE ? sizeof(c_t<T>) * (p.nsb - 1) * (KIND == SB_SPIN ? 3 : 1) * SX_T : 0);
+        if (sm > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        kern<<<grid, SX_T, sm, st>>>(p);
+        count_launches(1);
+    };
+    if constexpr (sizeof(T) == 4 && KIND == SB_DISP && LINE) {
+        // the SFU-bound case: no atom of weight zero up to six sites
+        switch (p.nsite) {
+        case 1: return go(k_sx_rows<T, KIND, 1, LINE, WGT>, 1);
+        case 2: return go(k_sx_rows<T, KIND, 2, LINE, WGT>, 2);
+        case 3: return go(k_sx_rows<T, KIND, 3, LINE, WGT>, 3);
+        case 5: return go(k_sx_rows<T, KIND, 5, LINE, WGT>, 5);
+        case 6: return go(k_sx_rows<T, KIND, 6, LINE, WGT>, 6);
+        default: break;
+        }
+    }
+    if constexpr (LINE) {
+        if (p.nsite <= 4) return go(k_sx_rows<T, KIND, 4, LINE, WGT>, 4);
+        if constexpr (sizeof(T) == 4)
+            if (p.nsite <= 8) return go(k_sx_rows<T, KIND, 8, LINE, WGT>, 8);
+    }
+    go(k_sx_rows<T, KIND, 16, LINE, WGT>, 16);
+}
+template <typename T, int KIND> void launch_rows(const SxParams<T> &p, bool line, const dim3 &grid, cudaStream_t st) {
+    if constexpr (KIND == SB_DISP) {
+        if (p.occ) return line ? launch_rows<T, KIND, true, true>(p, grid, st) : launch_rows<T, KIND, false, true>(p, grid, st);
+    }
+    return line ? launch_rows<T, KIND, true, false>(p, grid, st) : launch_rows<T, KIND, false, false>(p, grid, st);
+}
+
+template <typename T, int KIND> void run_kind(SxParams<T> p, double norm, int chunk_q, int nochunk, T *dout, cudaStream_t st) {
+    constexpr int NC = KIND == SB_SPIN ? 3 : 1;
+    const bool line = p.nsb <= SX_RING;
+    for (p.p0 = 0; p.p0 < p.npts; p.p0 += SX_PREP) {
+        p.np = std::min<long long>(SX_PREP, p.npts - p.p0);
+        k_sx_prep<T, KIND><<<(unsigned)((p.ldp + SX_T - 1) / SX_T), SX_T, 0, st>>>(p);
+        count_launches(1);
+        for (p.q0 = 0; p.q0 < p.np; p.q0 += chunk_q) {
+            p.nq = (int)std::min<long long>(chunk_q, p.np - p.q0);
+            const unsigned qb = (unsigned)((p.nq + SX_T - 1) / SX_T);
+            const dim3 rows(qb, (unsigned)p.nrb);
+            launch_rows<T, KIND>(p, line, rows, st);
+            if (!line) {
+                const size_t lines = (size_t)p.nmodels * p.ncell * NC;
+                k_sx_line<T><<<dim3(qb, (unsigned)std::min<size_t>(lines, 16384)), SX_T, 0, st>>>(p, NC);
+                count_launches(1);
+            }
+            if (KIND == SB_DISP && p.diffuse) {
+                k_sx_mean<T><<<dim3(qb * (SX_T / 32), (unsigned)p.nsite), 32 * SX_MB, 0, st>>>(p);
+                count_launches(1);
+            }
+            k_sx_boxes<T, KIND><<<dim3(qb, (unsigned)nochunk), SX_T, sizeof(int) * 2 * p.per_chunk * p.nsb, st>>>(p);
+            count_launches(1);
+        }
+    }
+    const unsigned nb = (unsigned)std::max<long long>(1, std::min<long long>((p.npts + 255) / 256, 152 * 8));
+    k_sx_sum<T><<<nb, 256, 0, st>>>(p.partial, p.npts, nochunk, norm, dout);
+    count_launches(1);
+}
+
+}  // namespace
+
+template <typename T>
+bool subbox_cells_run(ds_model *M, int kind, const SbSite *d_sites, const int4 *d_org, long long norigin,
+                      const double *d_hkl, long long npts, const ds_opts *o, T *dout, Scratch &ws, cudaStream_t st) {
+    using C = c_t<T>;
+    ds_ctx *ctx = M->ctx;
+    const int nsb = o->subbox_n, nsite = M->nsite, NC = kind == SB_SPIN ? 3 : 1;
+    const double cells = (double)M->nmodels * M->n[0] * M->n[1] * M->n[2];
+    // Rule: the cheaper route by a cost model, picoseconds per point, fitted to both routes measured in
+    // FP32 on GB300 (22,500 points; 1, 4 and 16 sites; 65 to 1040 boxes of 3^3 to 10^3 cells).  Box by
+    // box: per cell of a box 0.4 + 0.5 nsite (displacements), 0.9 + 0.145 nsite (occupancies), 0.66 +
+    // 0.5 nsite (moments), and the Debye-Waller pass of DIFFUSE displacements.  Shared: per cell 3.8 +
+    // 0.5, 2.2 + 0.28, 4.5 + 0.97 nsite, 0.9 per line sum read (0.9 per component), 2.3 per amplitude
+    // read where the line sums take their own pass.  fcc 32^3, n_sb = 5, 150 x 150 points: 520 origins
+    // 4.9 (box by box) and 4.4 ms, 260 origins 3.2 and 4.3 ms; occupancies 1040 origins 4.4 and 2.9 ms,
+    // 520 origins 2.3 and 2.7 ms.
+    double box_cell, cell;
+    if (kind == SB_DISP) box_cell = 0.4 + 0.5 * nsite, cell = 3.8 + 0.5 * nsite;
+    else if (kind == SB_OCC) box_cell = 0.9 + 0.145 * nsite, cell = 2.2 + 0.28 * nsite;
+    else box_cell = 0.66 + 0.5 * nsite, cell = 4.5 + 0.97 * nsite;
+    double by_box = (double)norigin * nsb * nsb * nsb * box_cell;
+    if (kind == SB_DISP && o->mode == DS_DIFFUSE) by_box += 0.48 * nsite * cells;
+    const double by_cell = cells * (cell + (nsb > SX_RING ? 2.3 * NC * nsb : 0.0)) + (double)norigin * nsb * nsb * 0.9 * NC;
+    if (by_cell > 0.95 * by_box) return false;
+    // points per chunk: line sums (and amplitudes, for boxes wider than the ring) within SX_L2
+    const size_t per_q = (size_t)cells * NC * sizeof(C) * (nsb > SX_RING ? 2 : 1);
+    long long blocks = std::max<long long>(1, (long long)(SX_L2 / (per_q * SX_T)));
+    blocks = std::min<long long>(blocks, (std::min<long long>(npts, SX_PREP) + SX_T - 1) / SX_T);
+    const int chunk_q = (int)blocks * SX_T;
+    if ((size_t)chunk_q * per_q > SX_MOST) return false;
+    SxParams<T> p;
+    memset(&p, 0, sizeof(p));
+    p.nsite = nsite;
+    p.nsb = nsb;
+    p.n1 = M->n[0];
+    p.n2 = M->n[1];
+    p.n3 = M->n[2];
+    p.ncell = p.n1 * p.n2 * p.n3;
+    p.nmodels = M->nmodels;
+    p.diffuse = o->mode == DS_DIFFUSE;
+    p.site = d_sites;
+    p.occ = (kind == SB_OCC || (kind == SB_DISP && M->has_occ)) ? M->d_occ : nullptr;
+    p.vec = kind == SB_SPIN ? M->d_spins : M->d_disp;
+    p.mean = kind == SB_OCC ? (M->user_mean ? M->d_user_mean : M->d_mean_occ) : M->d_mean_spin;
+    p.hkl = d_hkl;
+    p.npts = npts;
+    p.ld = chunk_q;
+    // a chunk's last block may reach past the held points: the constants are padded by one chunk
+    p.ldp = (std::min<long long>(npts, SX_PREP) + chunk_q - 1) / chunk_q * chunk_q;
+    p.origins = d_org;
+    p.norigin = norigin;
+    for (int i = 0; i < 9; ++i) p.recip[i] = M->recip[i];
+    // row blocks: about eight blocks per SM
+    const long long nrow = (long long)p.nmodels * p.n1 * p.n2;
+    const long long want = std::max<long long>(1, 152 * 8 / blocks);
+    p.rows_per = (int)std::max<long long>(1, (nrow + want - 1) / want);
+    if (nrow > (1LL << 31) - 1 || (nrow + p.rows_per - 1) / p.rows_per > 65535) return false;
+    p.nrb = (int)((nrow + p.rows_per - 1) / p.rows_per);
+    // origins per block: about eight blocks per SM, their row offsets within 32 KB of shared memory
+    p.per_chunk = std::min<long long>(std::max<long long>(1, (norigin + want - 1) / want), 4096 / nsb);
+    if ((norigin + p.per_chunk - 1) / p.per_chunk > 65535) return false;
+    const int nochunk = (int)((norigin + p.per_chunk - 1) / p.per_chunk);
+    const size_t nk = (size_t)p.ldp, before = ws.total;
+    const size_t need = sizeof(C) * nk * (nsite + 3 + 1 + NC) + sizeof(T) * 3 * nk + (size_t)chunk_q * per_q +
+                        (kind == SB_DISP && p.diffuse ? sizeof(T) * (size_t)(p.nrb + 1) * nsite * p.ld : 0) +
+                        sizeof(T) * (size_t)nochunk * npts;
+    if (before + need > ctx->budget) return false;
+    p.phi = (C *)ws.get(sizeof(C) * nk * nsite);
+    p.e = (C *)ws.get(sizeof(C) * nk * 3);
+    p.Q = (T *)ws.get(sizeof(T) * nk * 3);
+    p.B = (C *)ws.get(sizeof(C) * nk);
+    p.K = (C *)ws.get(sizeof(C) * nk * NC);
+    p.L = (C *)ws.get(sizeof(C) * (size_t)cells * NC * p.ld);
+    if (nsb > SX_RING) p.A = (C *)ws.get(sizeof(C) * (size_t)cells * NC * p.ld);
+    if (kind == SB_DISP && p.diffuse) {
+        p.dwp = (T *)ws.get(sizeof(T) * (size_t)(p.nrb + 1) * nsite * p.ld);
+        p.dwm = p.dwp + (size_t)p.nrb * nsite * p.ld;
+    }
+    p.partial = (T *)ws.get(sizeof(T) * (size_t)nochunk * npts);
+    if (ws.failed) {
+        ws.failed = false;   // the box-by-box route needs less
+        return false;
+    }
+    double norm = 1.0 / ((double)norigin * nsite * (double)nsb * nsb * nsb);
+    if (kind == SB_SPIN) norm *= 0.07265;  // C of Eq. mag_intensity (barn)
+    ProfScope ps(ctx, "subbox_cells", st);
+    if (kind == SB_OCC) run_kind<T, SB_OCC>(p, norm, chunk_q, nochunk, dout, st);
+    else if (kind == SB_SPIN) run_kind<T, SB_SPIN>(p, norm, chunk_q, nochunk, dout, st);
+    else run_kind<T, SB_DISP>(p, norm, chunk_q, nochunk, dout, st);
+    return true;
+}
+
+template bool subbox_cells_run<float>(ds_model *, int, const SbSite *, const int4 *, long long, const double *, long long,
+                                      const ds_opts *, float *, Scratch &, cudaStream_t);
+template bool subbox_cells_run<double>(ds_model *, int, const SbSite *, const int4 *, long long, const double *,
+                                       long long, const ds_opts *, double *, Scratch &, cudaStream_t);

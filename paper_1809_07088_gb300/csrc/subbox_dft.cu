@@ -30,6 +30,7 @@
 #include <vector>
 
 #include "api_internal.h"
+#include "subbox_points.h"
 
 using namespace ds;
 
@@ -39,17 +40,6 @@ constexpr int SB_THREADS = 128;
 constexpr int SB_STAGE = 2048;   // atoms staged per pass (float4: 32 KB)
 constexpr int DW_THREADS = 128;
 constexpr int DW_STAGE = 1024;
-enum { SB_OCC = 0, SB_SPIN = 1, SB_DISP = 2 };
-
-// per-site constants of the sub-box sum (FP64, built on the host)
-struct SbSite {
-    double r[3];
-    double b;
-    double coef[9];
-    int kind;
-    int pad;
-};
-
 template <typename T> struct SbParams {
     int nsite, nsb, n1, n2, n3, ncell;
     int diffuse;
@@ -65,35 +55,6 @@ template <typename T> struct SbParams {
     double recip[9];       // a*, b*, c* rows (1/A, 2 pi included)
     T *partial;            // [chunk][npts]
 };
-
-// Phases are carried in cycles (Q.x / 2 pi) and brought to [-1/2, 1/2] by subtracting the
-// nearest integer before the sine and cosine, where the fast FP32 __sincosf / __cosf are
-// accurate; FP64 uses sincospi / cospi.
-// x minus its nearest integer.  FP32: adding and subtracting 1.5 * 2^23 rounds |x| < 2^22 to
-// the nearest integer on the FMA pipe (rintf would take a slot of the SFU/conversion pipe that
-// the sine and cosine need); phases here are a few cycles.
-__device__ __forceinline__ double frac_w(double x) { return x - rint(x); }
-__device__ __forceinline__ float frac_w(float x) {
-    const float r = __fsub_rn(__fadd_rn(x, 12582912.0f), 12582912.0f);
-    return __fsub_rn(x, r);
-}
-// cos 2 pi t for a phase t in cycles (reduced to [-1/2, 1/2] first)
-__device__ __forceinline__ double cos_cycles(double t) { return cospi(2.0 * frac_w(t)); }
-__device__ __forceinline__ float cos_cycles(float t) { return __cosf(frac_w(t) * 6.283185307179586f); }
-// (cos 2 pi r, sin 2 pi r) for |r| <= 1/2
-__device__ __forceinline__ void sincos_cycles(double r, double &c, double &s) { sincospi(2.0 * r, &s, &c); }
-__device__ __forceinline__ void sincos_cycles(float r, float &c, float &s) { __sincosf(r * 6.283185307179586f, &s, &c); }
-// S += phi (c + i s) = phi c + (i phi) s: two paired FP32 multiply-adds
-__device__ __forceinline__ void cexp_acc(float2 &S, float2 phi, float2 iphi, float c, float s) {
-    S = __ffma2_rn(phi, make_float2(c, c), S);
-    S = __ffma2_rn(iphi, make_float2(s, s), S);
-}
-__device__ __forceinline__ void cexp_acc(double2 &S, double2 phi, double2 iphi, double c, double s) {
-    S.x = fma(phi.x, c, S.x);
-    S.x = fma(iphi.x, s, S.x);
-    S.y = fma(phi.y, c, S.y);
-    S.y = fma(iphi.y, s, S.y);
-}
 
 // Occupational and magnetic boxes: per cell, the site sum sum_mu phi_mu (a - abar) times the
 // cell phase exp(2 pi i Q.d), advanced by one complex multiply per cell.
@@ -820,16 +781,23 @@ ds_status run_subbox_points(ds_model *Mdl, const std::vector<int4> &org, const d
     int4 *d_org = (int4 *)ws.get(sizeof(int4) * norigin);
     const double *d_hkl = hkl;
     if (!hkl_dev) d_hkl = (const double *)ws.get(sizeof(double) * 3 * npts);
-    T *partial = (T *)ws.get(sizeof(T) * nchunk * npts);
-    T *dw = (kind == SB_DISP && o->mode == DS_DIFFUSE) ? (T *)ws.get(sizeof(T) * nsite * npts) : nullptr;
     T *dout = out_dev ? (T *)out : (T *)ws.get(sizeof(T) * npts);
     if (ws.failed) return ds_fail(ctx, DS_ERR_OOM, "device allocation failed (sub-box points)");
-    if (ws.total > ctx->budget)
-        return ds_fail(ctx, DS_ERR_ADMISSION, "request needs %zu bytes of scratch, budget %zu", ws.total, ctx->budget);
+    // the box-by-box route's buffers count against the budget whichever route runs
+    const size_t by_box = sizeof(T) * nchunk * npts + (kind == SB_DISP && o->mode == DS_DIFFUSE ? sizeof(T) * nsite * npts : 0);
+    if (ws.total + by_box > ctx->budget)
+        return ds_fail(ctx, DS_ERR_ADMISSION, "request needs %zu bytes of scratch, budget %zu", ws.total + by_box, ctx->budget);
     if (cudaMemcpyAsync(d_sites, sites.data(), sizeof(SbSite) * nsite, cudaMemcpyHostToDevice, st) != cudaSuccess ||
         cudaMemcpyAsync(d_org, org.data(), sizeof(int4) * norigin, cudaMemcpyHostToDevice, st) != cudaSuccess ||
         (!hkl_dev && cudaMemcpyAsync((void *)d_hkl, hkl, sizeof(double) * 3 * npts, cudaMemcpyHostToDevice, st) != cudaSuccess))
         return ds_fail(ctx, DS_ERR_CUDA, "copy of the sub-box inputs failed");
+    T *partial = nullptr, *dw = nullptr;
+    const bool shared = subbox_cells_run<T>(Mdl, kind, d_sites, d_org, norigin, d_hkl, npts, o, dout, ws, st);
+    if (!shared) {
+        partial = (T *)ws.get(sizeof(T) * nchunk * npts);
+        if (kind == SB_DISP && o->mode == DS_DIFFUSE) dw = (T *)ws.get(sizeof(T) * nsite * npts);
+        if (ws.failed) return ds_fail(ctx, DS_ERR_OOM, "device allocation failed (sub-box points)");
+    }
     if (dw) {
         ProfScope ps(ctx, "debye_waller", st);
         DwParams<T> d = dw_params<T>(Mdl, true);
@@ -861,7 +829,7 @@ ds_status run_subbox_points(ds_model *Mdl, const std::vector<int4> &org, const d
     p.per_chunk = per;
     for (int i = 0; i < 9; ++i) p.recip[i] = Mdl->recip[i];
     p.partial = partial;
-    {
+    if (!shared) {
         ProfScope ps(ctx, "subbox_dft", st);
         kern<<<dim3((unsigned)pblocks, (unsigned)nchunk), SB_THREADS, 0, st>>>(p);
         double norm = 1.0 / ((double)norigin * nsite * (double)p.nsb * p.nsb * p.nsb);

@@ -54,3 +54,23 @@ def test_debye_waller_grid_routes(ctx, prec, tag, sigma, count):
     want = core.magnetic_intensity_fft(m, m.qgrid.g_index(m.cells), 0, dw=True)
     scale = np.max(core.magnetic_intensity_fft(m, m.qgrid.g_index(m.cells), 0))
     assert np.max(np.abs(got.reshape(-1) - want)) / scale < TOL[tag]
+
+
+@pytest.mark.parametrize("prec,tag", PREC)
+@pytest.mark.parametrize("kind", ["occ", "spin", "disp"])
+@pytest.mark.parametrize("cells,nsb,nsite,npts,mode", [((6, 5, 4), 4, 3, 130, 1), ((6, 5, 4), 3, 5, 128, 0),
+                                                       ((4, 7, 8), 4, 1, 1, 1), ((9, 10, 9), 9, 1, 9, 1)])
+def test_subbox_points_shared_cell_amplitudes(ctx, prec, tag, kind, cells, nsb, nsite, npts, mode):
+    """Overlapping boxes at many origins (cell amplitudes shared by the boxes, rows of cells that wrap,
+    a remainder of points, boxes as wide as a row and wider than the register ring) against the
+    brute-force sum over boxes; occupancy weights with the displacements."""
+    code = {"occ": syn.OCC, "spin": syn.SPIN, "disp": syn.DISP}[kind]
+    nm = 1 if nsb > 8 else 2
+    m = syn.small_case(code, cells=cells, nsite=nsite, nmodels=nm, seed=233)
+    lm = to_library(ctx, m)
+    rng = np.random.default_rng(11)
+    hkl = rng.uniform(-1.7, 1.7, (npts, 3))
+    org = syn.random_origins(rng, nm, cells, 3 * nm * int(np.prod(cells)) // (8 if nsb > 8 else 1))
+    got, _ = lm.subbox_points(hkl, org, disorder=code, mode=mode, precision=prec, subbox_n=nsb)
+    want = noise.subbox_intensity(m, kind, mode, nsb, hkl, org)
+    assert rel_err_of_peak(got, want) < TOL[tag]
