@@ -1243,6 +1243,10 @@ extern "C" ds_status ds_request_intensity(ds_model *M, const ds_qgrid *q, const 
     return run_intensity<float>(M, q, o, out, out_is_device, st, info);
 }
 
+template ds_status site_tables<float>(ds_model *, const Geometry &, const GridMap &, int, int, cudaStream_t, Scratch &,
+                                      const c_t<float> **, const c_t<float> **);
+template ds_status site_tables<double>(ds_model *, const Geometry &, const GridMap &, int, int, cudaStream_t, Scratch &,
+                                       const c_t<double> **, const c_t<double> **);
 template ds_status plan_and_run<float>(ds_model *, const ds_qgrid *, const ds_opts *, float *, cudaStream_t,
                                        Scratch &, ds_result_info *, ForwardKeep<float> *, const TaylorHint *);
 template ds_status plan_and_run<double>(ds_model *, const ds_qgrid *, const ds_opts *, double *, cudaStream_t,

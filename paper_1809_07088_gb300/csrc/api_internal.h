@@ -164,6 +164,10 @@ ds_status taylor_order_from_corners(ds_ctx *ctx, const ds_opts *o, const double 
                                     double *umax);
 size_t request_footprint(const ds_model *M, const ds_qgrid *q, const ds_opts *o, int P);
 bool residue_classes(const ds_model *M, const ds::GridMap &gm, int dres[3]);
+// site phase tables of a grid, cached per model (api.cu)
+template <typename T>
+ds_status site_tables(ds_model *M, const ds::Geometry &g, const ds::GridMap &gm, int nmax, int nHmax, cudaStream_t st,
+                      Scratch &ws, const ds::c_t<T> **phk, const ds::c_t<T> **phH);
 // Lanczos resampling with the separable or the spherical cutoff (api.cu)
 bool lanczos_like(const ds_opts *o);
 double sphere_cutoff_radius(const ds_model *M, int m, int mprime);

@@ -74,3 +74,20 @@ def test_subbox_points_shared_cell_amplitudes(ctx, prec, tag, kind, cells, nsb, 
     got, _ = lm.subbox_points(hkl, org, disorder=code, mode=mode, precision=prec, subbox_n=nsb)
     want = noise.subbox_intensity(m, kind, mode, nsb, hkl, org)
     assert rel_err_of_peak(got, want) < TOL[tag]
+
+
+@pytest.mark.parametrize("prec,tag", PREC)
+@pytest.mark.parametrize("kind,cells,nsb,nm", [("occ", (2, 3, 2), 1, 2), ("spin", (5, 4, 7), 2, 2), ("occ", (16, 18, 21), 8, 1),
+                                               ("occ", (18, 20, 18), 9, 1)])
+def test_subbox_correlations_by_planes(ctx, prec, tag, kind, cells, nsb, nm):
+    """Windowed pair correlations of every box width: one cell, rows that are not multiples of four, more
+    rows than row lanes, the widest box of the plane kernel and one beyond it, against the brute-force
+    sum over boxes."""
+    code = {"occ": syn.OCC, "spin": syn.SPIN}[kind]
+    count = (3, 2, 4) if max(cells) > 8 else (7, 5, 6)
+    grid = syn.QGrid(h0=tuple(-2.0 / n for n in cells), step=tuple(1.0 / n for n in cells), count=count)
+    m = syn.small_case(code, cells=cells, nsite=2, nmodels=nm, seed=234, qgrid=grid)
+    lm = to_library(ctx, m)
+    got, _ = lm.intensity(qgrid_tuple(grid), disorder=code, mode=1, precision=prec, smoothing=2, subbox_n=nsb)
+    want = noise.subbox_intensity(m, kind, 1, nsb, grid.hkl())
+    assert rel_err_of_peak(got, want) < TOL[tag]
