@@ -51,6 +51,34 @@ struct FieldSource {
     const void *real_buf; // SRC_REAL: [field][cell] (T)
 };
 
+// Spectra of occupancy and spin fields: [field][k] (k < ncell_h).  Spectra of Taylor monomials:
+// [model][site][k / 32][monomial][k % 32].  The recombination reads every monomial of one k: with the
+// field index outermost these are reads one field (1 MB at 64^3) apart, each on a page of its own, at
+// about 10^10 a second on GB300 whatever their width; with 32 k in the innermost run they lie within
+// 1.4 MB (5456 monomials), and the transforms still store whole 256-byte runs.
+// perovskite 64^3, order 30 (5 x 5456 fields): recombination 90.3 -> 76.3 ms, transforms 29.6 -> 29.2 ms;
+// fcc 32^3 (4 x 5456 fields): 4.75 -> 4.40 ms, 1.90 -> 1.98 ms.
+constexpr int SPEC_KB = 32;
+__host__ __device__ __forceinline__ size_t disp_spec_site(int ncell_h, int nT) {   // elements per (model, site)
+    return (size_t)((ncell_h + SPEC_KB - 1) / SPEC_KB) * SPEC_KB * nT;
+}
+__host__ __device__ __forceinline__ size_t disp_spec_k(int kidx, int nT) {   // of monomial 0; SPEC_KB apart
+    return (size_t)(kidx / SPEC_KB) * SPEC_KB * nT + (kidx & (SPEC_KB - 1));
+}
+// where a field's transform is stored
+template <typename C> struct SpecOut {
+    C *base;
+    size_t blk;   // elements from one block of k to the next (0: plain)
+    __device__ __forceinline__ C &at(int kidx) const {
+        return blk ? base[(size_t)(kidx / SPEC_KB) * blk + (kidx & (SPEC_KB - 1))] : base[kidx];
+    }
+};
+template <typename C> __device__ __forceinline__ SpecOut<C> spec_out(const FieldSource &src, C *spec, int f, int ncell_h) {
+    if (src.kind != SRC_DISP) return {spec + (size_t)f * ncell_h, 0};
+    const int ms = f / src.T, t = f - ms * src.T;
+    return {spec + (size_t)ms * disp_spec_site(ncell_h, src.T) + (size_t)t * SPEC_KB, (size_t)src.T * SPEC_KB};
+}
+
 // output grid in supercell indices G_alpha = g0_alpha + i_alpha, split into zones H
 struct GridMap {
     int g0[3];

@@ -900,7 +900,7 @@ __global__ void __launch_bounds__(DISP_KT * 32, MINB) k_recomb_disp(const __grid
             const int ki = kidx_s[kk];
             if (tt < tc && ki >= 0 && s < nsite) {
                 const int t = tmap ? tmap[t0 + tt] : t0 + tt;
-                cp_async<sizeof(C)>(d, p.spec + (((size_t)p.model * nsite + site_s[s]) * nT + t) * g.ncell_h + ki);
+                cp_async<sizeof(C)>(d, p.spec + ((size_t)p.model * nsite + site_s[s]) * disp_spec_site(g.ncell_h, nT) + disp_spec_k(ki, nT) + (size_t)t * SPEC_KB);
             } else {
                 *d = mk<T>(T(0), T(0));
             }
@@ -1023,10 +1023,11 @@ __global__ void k_avg0(int nmodels, int nsite, int nT, int ncell_h, const int4 *
                        c_t<T> *avg0) {
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= nsite * nT) return;
-    const int t = idx % nT;
+    const int s = idx / nT, t = idx - s * nT;
     c_t<T> acc = mk<T>(T(0), T(0));
     if ((terms[t].w & 1) == 0)
-        for (int m = 0; m < nmodels; ++m) acc = cadd(acc, spec[((size_t)m * nsite * nT + idx) * ncell_h]);
+        for (int m = 0; m < nmodels; ++m)
+            acc = cadd(acc, spec[((size_t)m * nsite + s) * disp_spec_site(ncell_h, nT) + (size_t)t * SPEC_KB]);
     avg0[idx] = cscale(acc, T(1) / T(nmodels));
 }
 
