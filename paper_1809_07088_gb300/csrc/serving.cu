@@ -336,8 +336,14 @@ extern "C" ds_status ds_submit(ds_model *M, const ds_qgrid *q, const ds_opts *o,
     return DS_OK;
 }
 
-// fills info of a finished job, returns its status and forgets it
-static ds_status finish(ds_ctx *ctx, ServeJob *j, ds_result_info *info) {
+// fills info of a finished job, returns its status and forgets it.  The job leaves the table under the
+// lock and its events are read and destroyed after the lock is released: a completion callback waits
+// for ctx->mu, and a driver call of another thread (an allocation, a launch that has to resize local
+// memory) may wait for that callback with the driver's own lock held, so a thread that called the
+// driver while holding ctx->mu could close the circle.
+static ds_status finish(ds_ctx *ctx, ServeJob *j, ds_result_info *info, std::unique_lock<std::mutex> &lk) {
+    ctx->jobs.erase(j->ticket);
+    lk.unlock();
     ds_status st = j->status;
     if (info) {
         *info = j->info;
@@ -348,7 +354,6 @@ static ds_status finish(ds_ctx *ctx, ServeJob *j, ds_result_info *info) {
     }
     cudaEventDestroy(j->e0);
     cudaEventDestroy(j->e1);
-    ctx->jobs.erase(j->ticket);
     delete j;
     return st;
 }
@@ -359,7 +364,7 @@ extern "C" ds_status ds_poll(ds_ctx *ctx, uint64_t ticket, ds_result_info *info)
     auto it = ctx->jobs.find(ticket);
     if (it == ctx->jobs.end()) return ds_fail(ctx, DS_ERR_ARG, "unknown ticket %llu", (unsigned long long)ticket);
     if (!it->second->done) return DS_ERR_STATE;
-    return finish(ctx, it->second, info);
+    return finish(ctx, it->second, info, lk);
 }
 
 extern "C" ds_status ds_wait(ds_ctx *ctx, uint64_t ticket, double timeout_s, ds_result_info *info) {
@@ -371,7 +376,7 @@ extern "C" ds_status ds_wait(ds_ctx *ctx, uint64_t ticket, double timeout_s, ds_
     const auto deadline = std::chrono::steady_clock::now() + std::chrono::duration<double>(timeout_s > 0 ? timeout_s : 0);
     if (!ctx->cv.wait_until(lk, deadline, [&] { return j->done; }))
         return ds_fail(ctx, DS_ERR_TIMEOUT, "ticket %llu not finished after %.3f s", (unsigned long long)ticket, timeout_s);
-    return finish(ctx, j, info);
+    return finish(ctx, j, info, lk);
 }
 
 extern "C" ds_status ds_serving_pause(ds_ctx *ctx, int pause) {
