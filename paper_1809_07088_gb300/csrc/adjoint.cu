@@ -30,9 +30,9 @@ using namespace ds;
 
 namespace ds {
 // adjoint_sf.cu: Z of the displacive adjoint by the transposed sum factorisation (FP32); false when
-// it does not apply (order above 31, zone boxes wider than 17)
+// it does not apply (order above 31, zone boxes wider than 17).  half: the Hermitian part, stored half
 bool adjoint_z_disp_sf(const RecombParams<float> &p, const float *dLdI, const float2 *F, int P, double scale,
-                       float2 *Z, cudaStream_t s);
+                       float2 *Z, bool half, cudaStream_t s);
 }  // namespace ds
 
 namespace {
@@ -149,6 +149,96 @@ __global__ void __launch_bounds__(256) k_fft_columns_re32(int f0, int nf, const 
     T *o = out + (size_t)f * N * NC + c;
 #pragma unroll
     for (int k = 0; k < N; ++k) o[(size_t)k * NC] = cipow(a[k], rot).x;
+}
+
+// Real fields from stored half spectra (Hermitian by construction), i^rot folded in: the whole field in
+// one CTA's shared memory, lines in registers (the transpose of k_fft_field_reg): axis-1 columns
+// straight from global memory, axis-2 columns in place, then two rows per thread as one complex line
+// of axis 3 (Z = X + iY from their half spectra), staged for coalesced stores.
+template <int N> constexpr int fi_threads() { return N == 32 ? 544 : (N > 8 ? 1024 : 512); }   // 32: a thread per column
+template <typename T, int N>
+__global__ void __launch_bounds__(fi_threads<N>(), 1)
+    k_fft_field_inv(const c_t<T> *in, int f0, T *out, const int4 *terms, int nT) {
+    using C = c_t<T>;
+    constexpr int NH = N / 2 + 1, NROW = N * N, NPAIR = NROW / 2, NP = N + 1, NTH = fi_threads<N>();
+    static_assert(NPAIR <= NTH && N % 2 == 0, "one row pair per thread");
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    C *buf = (C *)smem_raw;      // [R1][k2][k3]
+    T *val = (T *)smem_raw;      // [row][NP]
+    static_assert(sizeof(T) * NROW * NP <= sizeof(C) * N * N * NH, "the rows fit the spectrum's buffer");
+    const int f = f0 + blockIdx.x, tid = threadIdx.x;
+    const int rot = terms ? terms[f % nT].w : 0;
+    const C *src = in + (size_t)f * N * N * NH;
+    for (int L = tid; L < N * NH; L += NTH) {
+        C y[N];
+#pragma unroll
+        for (int i = 0; i < N; ++i) y[i] = src[i * N * NH + L];
+        RegFFT<T, N>::run(y);
+#pragma unroll
+        for (int i = 0; i < N; ++i) buf[i * N * NH + L] = cipow(y[i], rot);
+    }
+    __syncthreads();
+    for (int L = tid; L < N * NH; L += NTH) {
+        const int r1 = L / NH, k3 = L - r1 * NH;
+        C *line = buf + r1 * N * NH + k3;
+        C y[N];
+#pragma unroll
+        for (int i = 0; i < N; ++i) y[i] = line[i * NH];
+        RegFFT<T, N>::run(y);
+#pragma unroll
+        for (int i = 0; i < N; ++i) line[i * NH] = y[i];
+    }
+    __syncthreads();
+    C z[N];
+    if (tid < NPAIR) {
+        const C *ra = buf + tid * NH, *rb = buf + (tid + NPAIR) * NH;
+#pragma unroll
+        for (int k = 0; k < NH; ++k) {
+            const C x = ra[k], y = rb[k];
+            if (k == 0 || k == N / 2) {
+                z[k] = mk<T>(x.x, y.x);              // real for Hermitian input
+            } else {
+                z[k] = mk<T>(x.x - y.y, x.y + y.x);          // X + iY
+                z[N - k] = mk<T>(x.x + y.y, y.x - x.y);      // conj X + i conj Y
+            }
+        }
+        RegFFT<T, N>::run(z);
+    }
+    __syncthreads();
+    if (tid < NPAIR) {
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            val[tid * NP + i] = z[i].x;
+            val[(tid + NPAIR) * NP + i] = z[i].y;
+        }
+    }
+    __syncthreads();
+    T *o = out + (size_t)f * N * N * N;
+    for (int i = tid; i < N * N * N; i += NTH) {
+        const int r = i / N;
+        o[i] = val[r * NP + (i - r * N)];
+    }
+}
+
+template <typename T, int N>
+void launch_field_inv(const c_t<T> *in, size_t nf, T *out, const int4 *terms, int nT, cudaStream_t s) {
+    constexpr size_t sm = (size_t)N * N * (N / 2 + 1) * sizeof(c_t<T>);
+    if (sm > 48 * 1024) cudaFuncSetAttribute(k_fft_field_inv<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    k_fft_field_inv<T, N><<<(unsigned)nf, fi_threads<N>(), sm, s>>>(in, 0, out, terms, nT);
+    count_launches(1);
+}
+
+// The adjoint's transforms end in Re[i^n sum_k exp(ik.R) Z(k)], so only the Hermitian part of i^n Z enters.
+// With F(-G) = conj F(G) and phi(-G) = conj phi(G) it is Z with dL/dI(G) replaced by the mean of
+// dL/dI(G) and dL/dI(-G): on a grid symmetric about the origin the stored half of the k suffices, half the
+// work and memory of Z, and a half-spectrum transform (cubic FP32 supercells of 8, 16, 20 or 32 cells).
+// fcc 32^3, 321^3 voxels, order 30: Z 9.75 -> 5.33 ms, transforms 3.33 -> 1.41 ms.
+bool adjoint_half(const Geometry &g, const int g0[3], const int cnt[3]) {
+    const int n = g.n[0];
+    if (g.n[1] != n || g.n[2] != n || !(n == 8 || n == 16 || n == 20 || n == 32)) return false;
+    for (int a = 0; a < 3; ++a)
+        if (g0[a] + (g0[a] + cnt[a] - 1) != 0) return false;
+    return true;
 }
 
 template <typename T>
@@ -370,31 +460,73 @@ struct GradAxes {
     double bg[9];  // gs_j b*_{j,alpha}, row j
 };
 
+// A block takes 64 cells of one (model, site) and eight slices of the exponents a (dealt in a snake order:
+// equal numbers of monomials); for each (a, b) the sum over c runs on values of D alone (two
+// multiply-adds per monomial, the powers of axis 3 in shared memory), the other powers enter once
+// per (a, b).  One thread per atom over every monomial left 1 CTA of 8 warps per SM waiting on
+// one load at a time: fcc 32^3, 5456 monomials: 2.40 -> 0.98 ms.
+constexpr int AG_CELLS = 64, AG_SLICES = 8;
 template <typename T>
-__global__ void k_adj_gather(int nmodels, int nsite, int ncell, int P, int nT, const int4 *terms, const T *pw,
-                             const uint8_t *occ, const T *D, const GradAxes ax, T *grad) {
-    const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const size_t natom = (size_t)nmodels * nsite * ncell;
-    if (idx >= natom) return;
-    const size_t ms = idx / ncell, cell = idx - ms * ncell;
+__global__ void __launch_bounds__(AG_CELLS * AG_SLICES)
+    k_adj_gather(int ncell, int P, int nT, const T *pw, const uint8_t *occ, const T *D, const GradAxes ax, T *grad) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T *pz_s = (T *)smem_raw;                                   // [e][cell]
+    T *red = pz_s + (size_t)(P + 1) * AG_CELLS;                // [slice][3][cell]
+    const int tx = threadIdx.x % AG_CELLS, ty = threadIdx.x / AG_CELLS;
+    const size_t ms = blockIdx.y;
+    const int cell = blockIdx.x * AG_CELLS + tx;
+    const bool live = cell < ncell;
+    const int cc = live ? cell : ncell - 1;
     const size_t P1 = (size_t)P + 1;
-    const T *px = pw + (ms * 3 + 0) * P1 * ncell + cell;
-    const T *py = pw + (ms * 3 + 1) * P1 * ncell + cell;
-    const T *pz = pw + (ms * 3 + 2) * P1 * ncell + cell;
-    const T *d = D + ms * (size_t)nT * ncell + cell;
+    const T *px = pw + (ms * 3 + 0) * P1 * ncell + cc;
+    const T *py = pw + (ms * 3 + 1) * P1 * ncell + cc;
+    const T *pz = pw + (ms * 3 + 2) * P1 * ncell + cc;
+    for (int e = ty; e <= P; e += AG_SLICES) pz_s[e * AG_CELLS + tx] = pz[(size_t)e * ncell];
+    __syncthreads();
+    const T *d0 = D + ms * (size_t)nT * ncell + cc;
     T gx = T(0), gy = T(0), gz = T(0);
-    for (int t = 0; t < nT; ++t) {
-        const int4 e = terms[t];
-        const T dv = d[(size_t)t * ncell];
-        const T ax = px[(size_t)e.x * ncell], by = py[(size_t)e.y * ncell], cz = pz[(size_t)e.z * ncell];
-        if (e.x > 0) gx = fma(dv, px[(size_t)(e.x - 1) * ncell] * by * cz, gx);
-        if (e.y > 0) gy = fma(dv, ax * py[(size_t)(e.y - 1) * ncell] * cz, gy);
-        if (e.z > 0) gz = fma(dv, ax * by * pz[(size_t)(e.z - 1) * ncell], gz);
+    for (int r = 0;; ++r) {
+        const int a = r * AG_SLICES + ((r & 1) ? AG_SLICES - 1 - ty : ty);
+        if (r * AG_SLICES > P) break;
+        if (a > P) continue;
+        const int q = P + 1 - a;
+        const int ta = ((P + 1) * (P + 2) * (P + 3) - q * (q + 1) * (q + 2)) / 6;   // monomials with a smaller a
+        const T xa = px[(size_t)a * ncell], xm = a > 0 ? px[(size_t)(a - 1) * ncell] : T(0);
+        const T *d = d0 + (size_t)ta * ncell;
+        T ym = T(0);
+        for (int b = 0; b <= P - a; ++b) {
+            const T yb = py[(size_t)b * ncell];
+            T s0 = T(0), s1 = T(0), zm = T(0);   // sums of D z^c / c! and of D z^(c-1) / (c-1)!
+            const int n = P - a - b + 1;
+#pragma unroll 8
+            for (int c = 0; c < n; ++c) {
+                const T dv = d[(size_t)c * ncell], z = pz_s[c * AG_CELLS + tx];
+                s0 = fma(dv, z, s0);
+                s1 = fma(dv, zm, s1);
+                zm = z;
+            }
+            d += (size_t)n * ncell;
+            gx = fma(xm * yb, s0, gx);
+            gy = fma(xa * ym, s0, gy);
+            gz = fma(xa * yb, s1, gz);
+            ym = yb;
+        }
     }
+    T *rd = red + (size_t)ty * 3 * AG_CELLS + tx;
+    rd[0] = gx, rd[AG_CELLS] = gy, rd[2 * AG_CELLS] = gz;
+    __syncthreads();
+    if (ty != 0 || !live) return;
+    T g[3];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        g[j] = T(0);
+        for (int sl = 0; sl < AG_SLICES; ++sl) g[j] += red[((size_t)sl * 3 + j) * AG_CELLS + tx];
+    }
+    const size_t idx = ms * ncell + cell;
     const T w = occ ? (T)occ[idx] : T(1);
 #pragma unroll
     for (int a = 0; a < 3; ++a)
-        grad[idx * 3 + a] = w * ((T)ax.bg[a] * gx + (T)ax.bg[3 + a] * gy + (T)ax.bg[6 + a] * gz);
+        grad[idx * 3 + a] = w * ((T)ax.bg[a] * g[0] + (T)ax.bg[3 + a] * g[1] + (T)ax.bg[6 + a] * g[2]);
 }
 
 template <typename T>
@@ -434,7 +566,8 @@ ds_status backward_run(ds_model *M, const ds_qgrid *q, const ds_opts *o, const T
     const double N = (double)nsite * g.ncell;
     const int nT = mag ? 3 : p.nT;
     const size_t nfield = (size_t)nmod * nsite * nT;
-    C *Z = (C *)ws.get(sizeof(C) * nfield * g.ncell);
+    C *Z = (C *)ws.get(sizeof(C) * nfield * g.ncell);   // half of it when the Hermitian part is formed
+    bool half = false;
     T *D = (T *)ws.get(sizeof(T) * nfield * g.ncell);
     const int fb = (int)std::max<size_t>(1, std::min<size_t>(nfield, (256ull << 20) / (sizeof(C) * (size_t)g.ncell)));
     C *work = (C *)ws.get(sizeof(C) * (size_t)fb * g.ncell);
@@ -448,7 +581,9 @@ ds_status backward_run(ds_model *M, const ds_qgrid *q, const ds_opts *o, const T
             bool done = false;
             if constexpr (sizeof(T) == 4) {
                 // FP32: the transposed sum factorisation over each k's zones (adjoint_sf.cu)
-                if (!mag) done = adjoint_z_disp_sf(p, dLdI, F, keep.src.P, 2.0 / (nmod * N), Z, st);
+                const bool h = !mag && adjoint_half(g, g0, cnt);
+                if (!mag) done = adjoint_z_disp_sf(p, dLdI, F, keep.src.P, 2.0 / (nmod * N), Z, h, st);
+                half = h && done;
             }
             if (done) {
             } else if (mag) {
@@ -478,22 +613,39 @@ ds_status backward_run(ds_model *M, const ds_qgrid *q, const ds_opts *o, const T
     }
     {
         ProfScope ps(ctx, "adjoint_fft", st);
-        for (size_t f0 = 0; f0 < nfield; f0 += fb)
+        if constexpr (sizeof(T) == 4) {
+            if (half) {
+                switch (g.n[0]) {
+                    case 8: launch_field_inv<T, 8>(Z, nfield, D, keep.terms, nT, st); break;
+                    case 16: launch_field_inv<T, 16>(Z, nfield, D, keep.terms, nT, st); break;
+                    case 20: launch_field_inv<T, 20>(Z, nfield, D, keep.terms, nT, st); break;
+                    default: launch_field_inv<T, 32>(Z, nfield, D, keep.terms, nT, st); break;
+                }
+            }
+        }
+        for (size_t f0 = 0; !half && f0 < nfield; f0 += fb)
             fft_complex_realpart<T>(g, Z, (int)f0, (int)std::min<size_t>(fb, nfield - f0), work, D, keep.W,
                                     mag ? nullptr : keep.terms, nT, st);
     }
     {
         ProfScope ps(ctx, "adjoint_gather", st);
-        const size_t natom = (size_t)nmod * nsite * g.ncell;
         if (mag) {
+            const size_t natom = (size_t)nmod * nsite * g.ncell;
             k_mag_grad_layout<T><<<(unsigned)((natom * 3 + 255) / 256), 256, 0, st>>>(nmod, nsite, g.ncell, D, grad);
         } else {
             GradAxes ax;
             for (int j = 0; j < 3; ++j)
                 for (int a = 0; a < 3; ++a) ax.bg[3 * j + a] = p.gscale[j] * p.recip[3 * j + a];
-            k_adj_gather<T><<<(unsigned)((natom + 255) / 256), 256, 0, st>>>(
-                nmod, nsite, g.ncell, keep.src.P, nT, keep.terms, keep.pw, M->has_occ ? M->d_occ : nullptr, D,
-                ax, grad);
+            const int P = keep.src.P;
+            const size_t sm = sizeof(T) * AG_CELLS * (P + 1 + 3 * AG_SLICES);
+            if (sm > 48 * 1024) cudaFuncSetAttribute(k_adj_gather<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+            // (model, site) pairs on the grid's y axis, at most 65535 per launch
+            for (int ms0 = 0; ms0 < nmod * nsite; ms0 += 65535) {
+                const int nms = std::min(65535, nmod * nsite - ms0);
+                const size_t at = (size_t)ms0 * g.ncell;
+                k_adj_gather<T><<<dim3((unsigned)((g.ncell + AG_CELLS - 1) / AG_CELLS), (unsigned)nms), AG_CELLS * AG_SLICES, sm, st>>>(
+                    g.ncell, P, nT, keep.pw + at * 3 * (P + 1), M->has_occ ? M->d_occ + at : nullptr, D + at * nT, ax, grad + at * 3);
+            }
         }
         count_launches(1);
     }

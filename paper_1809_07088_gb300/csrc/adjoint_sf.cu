@@ -12,7 +12,7 @@
 // with the powers of each axis tabulated once per k.  Each thread owns one output row of a step and
 // four consecutive powers (registers); every sum runs over the zones of one axis in a fixed order.
 //
-// CTA: one k of the full grid (the adjoint's complex FFT takes every k), shared memory sized for the
+// CTA: one k (of the full grid, or of the stored half for the Hermitian part: adjoint.cu), shared memory sized for the
 // widest zone box of the grid (zr zones per axis), 128, 256 or 512 threads as that footprint lets
 // 16 warps reside on an SM; per site the
 // zone factors beta are formed from gamma = scale dL/dI conj(F) (shared memory, once per k) and the
@@ -66,13 +66,14 @@ __host__ __device__ __forceinline__ AdjLayout adj_layout(int P, int zr) {
 template <int AS_THREADS>
 __global__ void __launch_bounds__(AS_THREADS, 512 / AS_THREADS)
     k_adj_taylor_sf(const __grid_constant__ RecombParams<float> p, const float *dLdI, const float2 *F, int P, int zr,
-                    float scale, float2 *Z) {
+                    float scale, int half, float2 *Z) {
     extern __shared__ __align__(16) unsigned char smem[];
     const Geometry &g = p.g;
     const GridMap &gm = p.gm;
     const int k = blockIdx.x;
     const int n1 = g.n[0], n2 = g.n[1], n3 = g.n[2];
-    const int kk[3] = {k / (n2 * n3), (k / n3) % n2, k % n3};
+    const int w3 = half ? g.n3h : n3;   // half: the stored half of the k (grid symmetric about the origin)
+    const int kk[3] = {k / (n2 * w3), (k / w3) % n2, k % w3};
     int lo[3], nz[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -82,7 +83,7 @@ __global__ void __launch_bounds__(AS_THREADS, 512 / AS_THREADS)
     }
     const int nsite = p.nsite, nT = p.nT, P1 = P + 1, P1p = (P1 + 3) & ~3;   // power rows padded to 4
     const int tid = threadIdx.x;
-    const size_t ncell = g.ncell;
+    const size_t ncell = half ? g.ncell_h : g.ncell;
     if (nz[0] * nz[1] * nz[2] == 0) {
         // no voxel of the grid has this k: every Z(k) is zero
         for (int i = tid; i < nsite * nT; i += AS_THREADS) {
@@ -117,7 +118,8 @@ __global__ void __launch_bounds__(AS_THREADS, 512 / AS_THREADS)
         const int G1 = n1 * (lo[0] + j) + kk[0], G2 = n2 * (lo[1] + h2) + kk[1], G3 = n3 * (lo[2] + h3) + kk[2];
         const size_t v = ((size_t)(G1 - gm.g0[0]) * gm.cnt[1] + (G2 - gm.g0[1])) * gm.cnt[2] + (G3 - gm.g0[2]);
         const float2 Fv = F[(size_t)p.model * nv + v];
-        float gI = dLdI[v] * scale;
+        // half: the Hermitian part of Z takes the mean over G and -G
+        float gI = (half ? 0.5f * (dLdI[v] + dLdI[nv - 1 - v]) : dLdI[v]) * scale;
         if (p.ff.ncls == 1) {
             // one form-factor class: f(|G|) enters every beta of the zone, folded in here once
             float Q[3];
@@ -240,7 +242,7 @@ __global__ void __launch_bounds__(AS_THREADS, 512 / AS_THREADS)
 }
 
 bool adjoint_z_disp_sf(const RecombParams<float> &p, const float *dLdI, const float2 *F, int P, double scale,
-                       float2 *Z, cudaStream_t s) {
+                       float2 *Z, bool half, cudaStream_t s) {
     if (P > AS_PMAX) return false;
     // widest zone box of any k along any axis
     int zr = 1;
@@ -253,19 +255,19 @@ bool adjoint_z_disp_sf(const RecombParams<float> &p, const float *dLdI, const fl
     if (zr > AS_ZR) return false;
     const AdjLayout L = adj_layout(P, zr);
     if (L.total > 227 * 1024) return false;
-    const unsigned nb = (unsigned)p.g.ncell;
+    const unsigned nb = (unsigned)(half ? p.g.ncell_h : p.g.ncell);
     switch (sf_threads_for(L.total)) {
         case 128:
             cudaFuncSetAttribute(k_adj_taylor_sf<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total);
-            k_adj_taylor_sf<128><<<nb, 128, L.total, s>>>(p, dLdI, F, P, zr, (float)scale, Z);
+            k_adj_taylor_sf<128><<<nb, 128, L.total, s>>>(p, dLdI, F, P, zr, (float)scale, half ? 1 : 0, Z);
             break;
         case 256:
             cudaFuncSetAttribute(k_adj_taylor_sf<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total);
-            k_adj_taylor_sf<256><<<nb, 256, L.total, s>>>(p, dLdI, F, P, zr, (float)scale, Z);
+            k_adj_taylor_sf<256><<<nb, 256, L.total, s>>>(p, dLdI, F, P, zr, (float)scale, half ? 1 : 0, Z);
             break;
         default:
             cudaFuncSetAttribute(k_adj_taylor_sf<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total);
-            k_adj_taylor_sf<512><<<nb, 512, L.total, s>>>(p, dLdI, F, P, zr, (float)scale, Z);
+            k_adj_taylor_sf<512><<<nb, 512, L.total, s>>>(p, dLdI, F, P, zr, (float)scale, half ? 1 : 0, Z);
             break;
     }
     count_launches(1);

@@ -273,8 +273,9 @@ __global__ void __launch_bounds__(512) k_fft_field(Geometry g, FieldSource src, 
 // One barrier per axis.
 // threads per CTA: at least one per row pair of axis 3 and one per line of axes 2 and 1; more
 // threads shorten the staging of the field values, which is bound by the latency of its loads
-// (20³ fields: 1024 threads stage in two rounds of loads instead of four)
-template <int N> constexpr int fr_threads() { return (N > 8 && N <= 20) ? 1024 : 512; }
+// (20³ fields: 1024 threads stage in two rounds of loads instead of four); 32³ fields: one thread per
+// line of axes 2 and 1 (32 x 17 = 544; with 512 a second round of one warp doubled both passes)
+template <int N> constexpr int fr_threads() { return N == 32 ? 544 : (N > 8 ? 1024 : 512); }
 
 template <typename T, int N1, int N2, int N3>
 __global__ void __launch_bounds__(fr_threads<N1>(), 1) k_fft_field_reg(const Geometry g, const FieldSource src, int f0,

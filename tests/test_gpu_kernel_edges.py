@@ -91,3 +91,19 @@ def test_subbox_correlations_by_planes(ctx, prec, tag, kind, cells, nsb, nm):
     got, _ = lm.intensity(qgrid_tuple(grid), disorder=code, mode=1, precision=prec, smoothing=2, subbox_n=nsb)
     want = noise.subbox_intensity(m, kind, 1, nsb, grid.hkl())
     assert rel_err_of_peak(got, want) < TOL[tag]
+
+
+@pytest.mark.parametrize("n,off", [(8, 0), (16, 0), (20, 0), (8, 1), (6, 0)])
+def test_displacive_adjoint_hermitian_part_and_full(ctx, n, off):
+    """FP32 gradient on grids symmetric about the origin (the Hermitian part of Z on the stored half of the
+    k, half-spectrum transform) and on a shifted or otherwise sized one (every k), against the FP64
+    gradient, with occupancy weights and a dL/dI that is not symmetric."""
+    m = syn.small_case(syn.DISP, cells=(n, n, n), nsite=3, nmodels=2, seed=235, sigma=0.08)
+    c = n + 3
+    m.qgrid = syn.QGrid(h0=tuple((off - c) / n for _ in range(3)), step=(1.0 / n,) * 3, count=(2 * c + 1,) * 3)
+    lm = to_library(ctx, m)
+    rng = np.random.default_rng(17)
+    d = rng.standard_normal(m.qgrid.count)
+    g64 = lm.backward(qgrid_tuple(m.qgrid), d, disorder=2, mode=0, precision=0, taylor_order=7)
+    g32 = lm.backward(qgrid_tuple(m.qgrid), d.astype(np.float32), disorder=2, mode=0, precision=1, taylor_order=7)
+    assert rel_err_of_peak(g32, g64) < 2e-5
