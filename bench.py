@@ -601,8 +601,9 @@ def taylor_sf_flops(cells, qgrid, P, nsite):
 
 
 def taylor_sf_adjoint_flops(cells, qgrid, P, nsite):
-    """Multiply-adds of the transposed sum factorisation of the adjoint: per k of the full grid and
-    per site, (P+1) n1 n2 n3 + (P+1)(P+2)/2 n2 n3 + T(P) n3 over the k's box of zones, 4 flop each."""
+    """Multiply-adds of the transposed sum factorisation of the adjoint: per k of the stored half (the
+    grid is symmetric about the origin) and per site, (P+1) n1 n2 n3 + (P+1)(P+2)/2 n2 n3 + T(P) n3
+    over the k's box of zones, 4 flop each."""
     import numpy as np
     n = list(cells)
     g0 = [int(round(qgrid.h0[a] * n[a])) for a in range(3)]
@@ -611,7 +612,7 @@ def taylor_sf_adjoint_flops(cells, qgrid, P, nsite):
     nab = (P + 1) * (P + 2) / 2.0
     nz = []
     for a in range(3):
-        k = np.arange(n[a])
+        k = np.arange(n[a] if a < 2 else n[a] // 2 + 1)
         lo = -((-(g0[a] - k)) // n[a])
         hi = (g0[a] + cnt[a] - 1 - k) // n[a]
         nz.append(np.maximum(hi - lo + 1, 0).astype(np.float64))
@@ -789,8 +790,8 @@ def run_rows(dev, cpu_rows=True):
     pts = torch.empty(hkl.shape[0], dtype=torch.float32, device=dev)
     ms, st = timed(lambda: ld.subbox_points(hkl, org, out=pts, disorder=ds.DS_DISP, mode=ds.DS_DIFFUSE,
                                             precision=ds.DS_FP32, subbox_n=5), reps=2)
-    terms = float(hkl.shape[0]) * org.shape[0] * 125 * md.nsite
-    sb = st.get("subbox_dft", float("nan"))
+    terms = float(hkl.shape[0]) * md.natom      # one per atom and point: the cells are shared by the boxes
+    sb = st.get("subbox_cells", float("nan"))
     mufu = alu["sfu_sincos_tops"] * 1e12   # (sin, cos) pairs per second, measured in this run
     rows["subbox_random_disp_fcc32_plane"] = {
         "workload": "fcc 32^3 displacive (u ~ N(0, 0.1^2)), %d random origins covering every cell, n_sb = 5, "
@@ -798,8 +799,8 @@ def run_rows(dev, cpu_rows=True):
         "ms": ms, "stages_ms": st, "points_per_s": hkl.shape[0] / (ms / 1e3),
         "roofline": {"bound": "alu", "achieved": terms / (sb / 1e3) / 1e12, "peak": mufu / 1e12,
                      "unit": "Tterm/s", "frac": terms / (sb / 1e3) / mufu,
-                     "note": "one exp(i Q.u) (one SFU sine-cosine pair) per atom, box and point; peak: "
-                             "__sincosf pairs per second measured in this run"}}
+                     "note": "one exp(i Q.u) (one SFU sine-cosine pair) per atom and point, cell amplitudes shared "
+                             "by the boxes; peak: __sincosf pairs per second measured in this run"}}
     ld.close()
 
     # magnetic + displacive coupling through T_mu(G) (Eq. mag_sf): pyrochlore 20^3, |hkl| <= 2
@@ -812,18 +813,15 @@ def run_rows(dev, cpu_rows=True):
     ms, st = timed(lambda: lmg.intensity(q, out=out, disorder=ds.DS_SPIN, mode=ds.DS_TOTAL, precision=ds.DS_FP32,
                                          dw_coupling=1), reps=2)
     dwms = st.get("debye_waller", float("nan"))
-    terms = float(mm.qgrid.nvox) * mm.nsite * mm.ncell
-    instr = 5.0 * terms                            # per term: 2 FFMA + 2 FMUL (rotation) + 1 FADD (sum)
-    fp32_instr = alu["fp32_fma_tflops"] / 2.0      # FP32 instructions per second (10^12)
+    dwb = 4.0 * mm.qgrid.nvox * mm.nsite + 12.0 * mm.natom   # factors written, displacements read
     rows["mag_dw_pyrochlore20"] = {
         "workload": "magnetic pyrochlore 20^3 with u ~ N(0, 0.05^2), |hkl| <= 2 step 1/20 (%d^3 voxels), "
                     "T_mu(G) per voxel and site, FP32" % mm.qgrid.count[0],
         "ms": ms, "stages_ms": st, "voxels_per_s": mm.qgrid.nvox / (ms / 1e3),
-        "roofline": {"bound": "alu", "achieved": instr / (dwms / 1e3) / 1e12, "peak": fp32_instr,
-                     "unit": "T FP32 instr/s", "frac": instr / (dwms / 1e3) / 1e12 / fp32_instr,
-                     "note": "Debye-Waller row recurrence: per voxel, site and lattice point one complex "
-                             "rotation and one add (5 FP32 instructions; the two sincos per 8 voxels left out); "
-                             "peak = measured FFMA rate"}}
+        "roofline": {"bound": "hbm", "achieved": dwb / (dwms / 1e3) / 1e9, "peak": hbm, "unit": "GB/s",
+                     "frac": dwb / (dwms / 1e3) / 1e9 / hbm,
+                     "note": "T_mu(G) from the moments of the displacements: factors written plus displacements "
+                             "read; five kernels, launch and FP64 latency at this size"}}
     lmg.close()
 
     # the displacive fcc 8^3 workload, plain FP64 (Taylor order by the remainder bound at eps 1e-8),
