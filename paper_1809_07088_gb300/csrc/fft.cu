@@ -189,11 +189,12 @@ __global__ void k_fft_columns(Geometry g, FieldSource src, int f0, int cb, const
         const int lf = f % src.nf_per_model;
         rot = src.terms[lf % src.T].w;
     }
-    const SpecOut<C> out = spec_out(src, spec, f, g.ncell_h);
-    for (int idx = threadIdx.x; idx < n1 * cb; idx += blockDim.x) {
-        const int k1 = (int)fcb.div((unsigned)idx), c = idx - k1 * cb;
-        if (c0 + c < ncol) out.at(k1 * ncol + c0 + c) = cipow(res[idx], rot);
-    }
+    spec_store(src, spec, f, g.ncell_h, [&](auto put) {
+        for (int idx = threadIdx.x; idx < n1 * cb; idx += blockDim.x) {
+            const int k1 = (int)fcb.div((unsigned)idx), c = idx - k1 * cb;
+            if (c0 + c < ncol) put(k1 * ncol + c0 + c, cipow(res[idx], rot));
+        }
+    });
 }
 
 // Whole-field variant for small supercells: one CTA holds every plane of one field in shared
@@ -257,11 +258,12 @@ __global__ void __launch_bounds__(512) k_fft_field(Geometry g, FieldSource src, 
         const int lf = f % src.nf_per_model;
         rot = src.terms[lf % src.T].w;
     }
-    const SpecOut<C> out = spec_out(src, spec, f, g.ncell_h);
-    for (int idx = threadIdx.x; idx < n1 * per_plane_h; idx += blockDim.x) {
-        const int k1 = (int)fph.div((unsigned)idx), rem = idx - k1 * per_plane_h;
-        out.at(idx) = cipow(res3[(size_t)k1 * plane_c + rem], rot);
-    }
+    spec_store(src, spec, f, g.ncell_h, [&](auto put) {
+        for (int idx = threadIdx.x; idx < n1 * per_plane_h; idx += blockDim.x) {
+            const int k1 = (int)fph.div((unsigned)idx), rem = idx - k1 * per_plane_h;
+            put(idx, cipow(res3[(size_t)k1 * plane_c + rem], rot));
+        }
+    });
 }
 
 // Whole field in shared memory with register-resident lines (sizes N1 x N2 x N3 known at compile
@@ -370,14 +372,15 @@ __global__ void __launch_bounds__(fr_threads<N1>(), 1) k_fft_field_reg(const Geo
     // axis 1: line (k2, k3), elements R1 N2 N3H apart; half spectrum to HBM
     int rot = 0;
     if (src.kind == SRC_DISP) rot = src.terms[(f % src.nf_per_model) % src.T].w;
-    const SpecOut<C> out = spec_out(src, spec, f, N1 * N2 * N3H);
     for (int L = tid; L < N2 * N3H; L += FR_THREADS) {
         C y[N1];
 #pragma unroll
         for (int i = 0; i < N1; ++i) y[i] = buf[i * N2 * N3H + L];
         RegFFT<T, N1>::run(y);
+        spec_store(src, spec, f, N1 * N2 * N3H, [&](auto put) {
 #pragma unroll
-        for (int i = 0; i < N1; ++i) out.at(i * N2 * N3H + L) = cipow(y[i], rot);
+            for (int i = 0; i < N1; ++i) put(i * N2 * N3H + L, cipow(y[i], rot));
+        });
     }
 }
 
@@ -595,12 +598,13 @@ __global__ void __launch_bounds__(C64_THREADS) k_fft_columns64(const FieldSource
         const int fl = (int)(b / NCH), c0 = (int)(b - (long long)fl * NCH) * CB, f = f0 + fl;
         int rot = 0;
         if (src.kind == SRC_DISP) rot = src.terms[(f % src.nf_per_model) % src.T].w;
-        const SpecOut<C> out = spec_out(src, spec, f, N * NCOL);
+        spec_store(src, spec, f, N * NCOL, [&](auto put) {
 #pragma unroll
-        for (int i = tid; i < N * CB; i += C64_THREADS) {
-            const int k1 = i >> 5, c = i & (CB - 1);
-            out.at(k1 * NCOL + c0 + c) = cipow(blk[k1 * CS + c], rot);
-        }
+            for (int i = tid; i < N * CB; i += C64_THREADS) {
+                const int k1 = i >> 5, c = i & (CB - 1);
+                put(k1 * NCOL + c0 + c, cipow(blk[k1 * CS + c], rot));
+            }
+        });
         __syncthreads();   // the buffer is free for the copies of the block after next
     }
 }

@@ -48,35 +48,39 @@ struct FieldSource {
     const void *pw;     // displacive powers (T) [model][site][3][P+1][cell]: (u Qs)^e / e!
     const int4 *terms;  // displacive monomials (a, b, c, n), lexicographic
     int T, P;           // number of monomials, order
+    int kb;             // layout of the monomials' spectra (SPEC_KB, or ncell_h: plain)
     const void *real_buf; // SRC_REAL: [field][cell] (T)
 };
 
-// Spectra of occupancy and spin fields: [field][k] (k < ncell_h).  Spectra of Taylor monomials:
-// [model][site][k / 32][monomial][k % 32].  The recombination reads every monomial of one k: with the
-// field index outermost these are reads one field (1 MB at 64^3) apart, each on a page of its own, at
-// about 10^10 a second on GB300 whatever their width; with 32 k in the innermost run they lie within
-// 1.4 MB (5456 monomials), and the transforms still store whole 256-byte runs.
-// perovskite 64^3, order 30 (5 x 5456 fields): recombination 90.3 -> 76.3 ms, transforms 29.6 -> 29.2 ms;
-// fcc 32^3 (4 x 5456 fields): 4.75 -> 4.40 ms, 1.90 -> 1.98 ms.
+// Spectra: [field][k] (k < ncell_h).  Taylor monomials whose spectra take more than SPEC_BLOCKED bytes:
+// [model][site][k / kb][monomial][k % kb], kb = SPEC_KB (kb = ncell_h is the plain layout).  The
+// recombination reads every monomial of one k: with the field index outermost these are reads one
+// field (1 MB at 64^3) apart, each on a page of its own, at about 10^10 a second on GB300 whatever
+// their width; with 32 k in the innermost run they lie within 1.4 MB (5456 monomials), and the
+// transforms still store whole 256-byte runs.  perovskite 64^3, order 30 (29.5 GB): recombination
+// 90.3 -> 76.3 ms, transforms 29.6 -> 29.2 ms; fcc 32^3 (3.0 GB): 4.75 -> 4.40 ms, 1.90 -> 1.98 ms.
+// Spectra near the size of the L2 gain nothing and the stores cost more (fcc 16^3, 130 MB: the volume
+// 493 us plain, 507 us blocked).
 constexpr int SPEC_KB = 32;
-__host__ __device__ __forceinline__ size_t disp_spec_site(int ncell_h, int nT) {   // elements per (model, site)
-    return (size_t)((ncell_h + SPEC_KB - 1) / SPEC_KB) * SPEC_KB * nT;
+constexpr size_t SPEC_BLOCKED = 512u << 20;
+__host__ __device__ __forceinline__ size_t disp_spec_site(int ncell_h, int nT, int kb) {   // elements per (model, site)
+    return (size_t)((ncell_h + kb - 1) / kb) * kb * nT;
 }
-__host__ __device__ __forceinline__ size_t disp_spec_k(int kidx, int nT) {   // of monomial 0; SPEC_KB apart
-    return (size_t)(kidx / SPEC_KB) * SPEC_KB * nT + (kidx & (SPEC_KB - 1));
+__host__ __device__ __forceinline__ size_t disp_spec_k(int kidx, int nT, int kb) {   // of monomial 0; kb apart
+    return (size_t)(kidx / kb) * kb * nT + kidx % kb;
 }
-// where a field's transform is stored
-template <typename C> struct SpecOut {
-    C *base;
-    size_t blk;   // elements from one block of k to the next (0: plain)
-    __device__ __forceinline__ C &at(int kidx) const {
-        return blk ? base[(size_t)(kidx / SPEC_KB) * blk + (kidx & (SPEC_KB - 1))] : base[kidx];
+// stores of a field's transform: store(put) with put(kidx, value), the layout chosen outside its loops
+template <typename C, typename F>
+__device__ __forceinline__ void spec_store(const FieldSource &src, C *spec, int f, int ncell_h, F &&store) {
+    if (src.kind != SRC_DISP || src.kb == ncell_h) {
+        C *base = spec + (size_t)f * ncell_h;
+        store([base](int kidx, const C &v) { base[kidx] = v; });
+    } else {
+        const int ms = f / src.T, t = f - ms * src.T;
+        C *base = spec + (size_t)ms * disp_spec_site(ncell_h, src.T, SPEC_KB) + (size_t)t * SPEC_KB;
+        const size_t blk = (size_t)src.T * SPEC_KB;
+        store([base, blk](int kidx, const C &v) { base[(size_t)(kidx / SPEC_KB) * blk + (kidx & (SPEC_KB - 1))] = v; });
     }
-};
-template <typename C> __device__ __forceinline__ SpecOut<C> spec_out(const FieldSource &src, C *spec, int f, int ncell_h) {
-    if (src.kind != SRC_DISP) return {spec + (size_t)f * ncell_h, 0};
-    const int ms = f / src.T, t = f - ms * src.T;
-    return {spec + (size_t)ms * disp_spec_site(ncell_h, src.T) + (size_t)t * SPEC_KB, (size_t)src.T * SPEC_KB};
 }
 
 // output grid in supercell indices G_alpha = g0_alpha + i_alpha, split into zones H
@@ -150,6 +154,7 @@ template <typename T> struct RecombParams {
     int nsite, nmodels, model;          // model: which supercell this launch handles
     int ncomp;                          // 1 (occupancy / displacive) or 3 (magnetic)
     int nT;                             // monomials per site (displacive)
+    int spec_kb;                        // layout of their spectra (see SPEC_KB)
     int accumulate;                     // add into out instead of overwriting
     int diffuse;
     const c_t<T> *spec;                 // [model][site][ncomp or T][ncell_h]

@@ -900,7 +900,7 @@ __global__ void __launch_bounds__(DISP_KT * 32, MINB) k_recomb_disp(const __grid
             const int ki = kidx_s[kk];
             if (tt < tc && ki >= 0 && s < nsite) {
                 const int t = tmap ? tmap[t0 + tt] : t0 + tt;
-                cp_async<sizeof(C)>(d, p.spec + ((size_t)p.model * nsite + site_s[s]) * disp_spec_site(g.ncell_h, nT) + disp_spec_k(ki, nT) + (size_t)t * SPEC_KB);
+                cp_async<sizeof(C)>(d, p.spec + ((size_t)p.model * nsite + site_s[s]) * disp_spec_site(g.ncell_h, nT, p.spec_kb) + disp_spec_k(ki, nT, p.spec_kb) + (size_t)t * p.spec_kb);
             } else {
                 *d = mk<T>(T(0), T(0));
             }
@@ -1019,7 +1019,7 @@ template <typename T> void recombine_disp(const RecombParams<T> &p, cudaStream_t
 
 // <F(H)> of Eq. bragg_sf_disp: even orders of the k = 0 transforms averaged over supercells
 template <typename T>
-__global__ void k_avg0(int nmodels, int nsite, int nT, int ncell_h, const int4 *terms, const c_t<T> *spec,
+__global__ void k_avg0(int nmodels, int nsite, int nT, int ncell_h, int kb, const int4 *terms, const c_t<T> *spec,
                        c_t<T> *avg0) {
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= nsite * nT) return;
@@ -1027,7 +1027,7 @@ __global__ void k_avg0(int nmodels, int nsite, int nT, int ncell_h, const int4 *
     c_t<T> acc = mk<T>(T(0), T(0));
     if ((terms[t].w & 1) == 0)
         for (int m = 0; m < nmodels; ++m)
-            acc = cadd(acc, spec[((size_t)m * nsite + s) * disp_spec_site(ncell_h, nT) + (size_t)t * SPEC_KB]);
+            acc = cadd(acc, spec[((size_t)m * nsite + s) * disp_spec_site(ncell_h, nT, kb) + (size_t)t * kb]);
     avg0[idx] = cscale(acc, T(1) / T(nmodels));
 }
 
@@ -1098,7 +1098,7 @@ __global__ void __launch_bounds__(256) k_bragg_disp(RecombParams<T> p, const c_t
 template <typename T>
 void displacive_bragg(const RecombParams<T> &p, const int4 *terms, c_t<T> *avg0, c_t<T> *bragg, cudaStream_t s) {
     const int n0 = p.nsite * p.nT;
-    k_avg0<T><<<(n0 + 255) / 256, 256, 0, s>>>(p.nmodels, p.nsite, p.nT, p.g.ncell_h, terms, p.spec, avg0);
+    k_avg0<T><<<(n0 + 255) / 256, 256, 0, s>>>(p.nmodels, p.nsite, p.nT, p.g.ncell_h, p.spec_kb, terms, p.spec, avg0);
     const int nz = p.gm.nH[0] * p.gm.nH[1] * p.gm.nH[2];
     int P = 0;   // the order of the nT monomials: (P + 1)(P + 2)(P + 3) / 6 = nT
     while ((P + 1) * (P + 2) * (P + 3) / 6 < p.nT) ++P;

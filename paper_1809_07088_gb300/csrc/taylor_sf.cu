@@ -197,12 +197,13 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_taylor_sf(const __grid_constan
     for (int i = tid; i < nzone; i += NT) Fs[i] = mk<T>(T(0), T(0));
     __syncthreads();
 
+    const size_t kb = p.spec_kb;   // from one monomial of a k to the next
     const bool one_ff = p.ff.ncls == 1;
     int cls = 0;
     for (int s = 0; s < nsite; ++s) {
         if (s == p.ff.cls_end[cls]) ++cls;
         const int site = p.site_of[s];
-        const C *spec_s = p.spec + (size_t)(p.model * nsite + site) * disp_spec_site(g.ncell_h, p.nT) + disp_spec_k(kidx, p.nT);
+        const C *spec_s = p.spec + (size_t)(p.model * nsite + site) * disp_spec_site(g.ncell_h, p.nT, p.spec_kb) + disp_spec_k(kidx, p.nT, p.spec_kb);
         for (int gi = pl.ngroups - 1; gi >= 0; --gi) {
             const int a0 = pl.a0[gi], a1 = pl.a0[gi + 1];
             // step 1: X[xi(a, b)][h3] = sum_c M'_abc x3^c, one (a, b) chain per slot
@@ -213,9 +214,9 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_taylor_sf(const __grid_constan
                 T x3[ZR];
 #pragma unroll
                 for (int j = 0; j < ZR; ++j) x3[j] = xs[2 * ZR + j];
-                const C *src = spec_s + (size_t)it.z * SPEC_KB;
+                const C *src = spec_s + (size_t)it.z * kb;
                 C acc[ZR];
-                const C top = src[(Lc - 1) * SPEC_KB];
+                const C top = src[(Lc - 1) * kb];
 #pragma unroll
                 for (int j = 0; j < ZR; ++j) acc[j] = top;
                 constexpr int NB = sizeof(T) == 4 ? 8 : 2;  // loads in flight per thread (registers)
@@ -223,7 +224,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_taylor_sf(const __grid_constan
                     C mb[NB];
 #pragma unroll
                     for (int q = 0; q < NB; ++q)
-                        if (c - q >= 0) mb[q] = src[(c - q) * SPEC_KB];
+                        if (c - q >= 0) mb[q] = src[(c - q) * kb];
 #pragma unroll
                     for (int q = 0; q < NB; ++q)
                         if (c - q >= 0) {
