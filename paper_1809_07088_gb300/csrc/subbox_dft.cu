@@ -459,11 +459,14 @@ __device__ __forceinline__ DwRoute dw_route(const double *xc, double eps, long l
         ++P;
         term *= x / (P + 1);
     }
+    // before P is made even: P = DW_PCAP + 1 is where the loop ends whether the bound was met there or not
+    const bool met = term <= eps;
     P = max(P & ~1, 2);   // odd orders do not enter; P >= 2 lets a non-finite displacement reach the sums
     const long long T2 = (long long)(P + 1) * (P + 2) * (P + 3) / 6;
     r.P = P;
-    // moments cost T2 / 2 products per lattice point, the direct sum one rotation per voxel and point
-    r.taylor = P <= DW_PCAP && T2 <= nvox;
+    // moments cost T2 / 2 products per lattice point, the direct sum one rotation per voxel and point; an
+    // x_max whose series needs more than DW_PCAP orders (above 6.6 in FP32, 3.3 in FP64) takes the direct sum
+    r.taylor = met && P <= DW_PCAP && T2 <= nvox;
     r.wide = eps < 1e-12 || x > 2.0;
     return r;
 }

@@ -1,0 +1,50 @@
+"""Rules that choose between two routes to one result, on both sides of each line, against the CPU FP64
+oracle (tolerances of the parity tests: 1e-10 of peak in FP64, 1e-5 in FP32)."""
+import numpy as np
+import pytest
+
+import synthetic as syn
+from oracle import core
+from _helpers import TOL, qgrid_tuple, to_library
+
+pytestmark = pytest.mark.gpu
+PREC = [(0, "fp64"), (1, "fp32")]
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    import paper_1809_07088_gb300 as ds
+    c = ds.Context(0)
+    yield c
+    c.close()
+
+
+def _dw_model(spread, xmax, count=(17, 17, 17)):
+    """Spins with displacements whose largest |Q.u| over the grid's corners is xmax: Gaussian ones, or
+    every atom at +u or -u (no voxel's mean is then carried by small arguments)."""
+    m = syn.small_case(syn.SPIN, cells=(6, 5, 4), nsite=3, nmodels=3, seed=241)
+    m.qgrid = syn.QGrid(h0=tuple(-(c // 2) / n for c, n in zip(count, m.cells)), step=tuple(1.0 / n for n in m.cells),
+                        count=count)
+    rng = np.random.default_rng(29)
+    if spread == "gauss":
+        u = rng.standard_normal(m.spins.shape)
+    else:
+        u = np.array([1.0, 0.7, -0.4]) * rng.choice([-1.0, 1.0], m.spins.shape[:-1])[..., None]
+    m.disp = u.astype(np.float32)
+    m.disp = (u * (xmax / core.x_max(m, m.qgrid))).astype(np.float32)
+    return m
+
+
+@pytest.mark.parametrize("spread", ["gauss", "pair"])
+@pytest.mark.parametrize("xmax", [1.9, 2.1, 3.1, 3.4, 5.0, 6.5, 6.7, 7.0, 10.0, 20.0])
+def test_debye_waller_grid_below_and_above_the_order_cap(ctx, spread, xmax):
+    """Grids of more voxels than the moments have monomials (4495 at order 28): |Q.u| below and above the
+    arguments whose series ends by that order (3.27 in FP64, 6.61 in FP32), where the direct sum serves."""
+    m = _dw_model(spread, xmax)
+    G = m.qgrid.g_index(m.cells)
+    want = core.magnetic_intensity_fft(m, G, 0, dw=True)
+    scale = np.max(core.magnetic_intensity_fft(m, G, 0))
+    lm = to_library(ctx, m)
+    for prec, tag in PREC:
+        got, _ = lm.intensity(qgrid_tuple(m.qgrid), disorder=1, mode=0, precision=prec, dw_coupling=1)
+        assert np.max(np.abs(got.reshape(-1) - want)) / scale < TOL[tag], tag
