@@ -436,8 +436,9 @@ template <typename T> struct DwParams {
 // voxel), the polynomial is evaluated axis by axis (P + 1 multiply-adds per voxel), in place of one
 // complex rotation per voxel and lattice point.  x_max stays on the device: k_dw_moments derives
 // the route from it for the kernels that follow, so the request needs no read-back; the direct kernel
-// returns at once when the moments serve.  Sums are taken in FP64 (partial sums of 16 terms in the working type); the
-// polynomial in the working type while x_max <= 2 (cosh x_max bounds the cancellation), else in FP64.
+// returns at once when the moments serve.  Sums are taken in FP64; the powers, products, partial sums of 16 terms and the
+// polynomial in the working type while x_max <= 2 (cosh x_max bounds the cancellation), else all in FP64: FP32
+// products left an error of T^2 of 1.2e-5 at x_max = 6.5 (every atom at +u or -u; 1.7e-8 in FP64).
 // 16 sites, 20^3 cells, 81^3 voxels, x_max about 0.5: the request takes 0.25 ms, 17.4 ms by the direct
 // sum (whose FP32 rotations left 1.6e-5 of the result; 1.1e-7 by the moments).  A grid of fewer voxels
 // than monomials keeps the direct sum: one rotation per voxel and point costs about a monomial's product.
@@ -477,21 +478,11 @@ __device__ __forceinline__ int dw_t0(int P, int a, int b) {
 }
 
 // part[chunk][site][t]: sums of v1^a v2^b v3^c / (a! b! c!) over the chunk's samples (even orders)
-template <typename T>
-__global__ void __launch_bounds__(256) k_dw_moments(const __grid_constant__ DwParams<T> p) {
-    __shared__ DwRoute rt;
-    if (threadIdx.x == 0) {
-        rt = dw_route(p.xc, dw_eps<T>(), p.npts);
-        if (blockIdx.x == 0 && blockIdx.y == 0) p.route[0] = rt.P, p.route[1] = rt.taylor, p.route[2] = rt.wide;
-    }
-    __syncthreads();
-    if (!rt.taylor) return;
-    const int P = rt.P, P1 = P + 1, s = blockIdx.y, ch = blockIdx.x;
+template <typename T, typename CT>
+__device__ __forceinline__ void dw_moments_body(const DwParams<T> &p, int P, CT *pw, CT *inv_e) {   // pw: [axis][e][sample]
+    const int P1 = P + 1, s = blockIdx.y, ch = blockIdx.x;
     constexpr int RS = DW_SUB + 1;                 // rows one apart in the banks
-    extern __shared__ __align__(16) unsigned char dw_raw[];
-    T *pw = (T *)dw_raw;                            // [axis][e][sample]
-    __shared__ T inv_e[DW_PCAP + 1];                // 1 / (e + 1)
-    if (threadIdx.x <= DW_PCAP) inv_e[threadIdx.x] = (T)(1.0 / (threadIdx.x + 1));
+    if (threadIdx.x <= DW_PCAP) inv_e[threadIdx.x] = (CT)(1.0 / (threadIdx.x + 1));
     const long long nsamp = (long long)p.nmodels * p.ncell;
     const long long per = (nsamp + p.nchunk - 1) / p.nchunk;
     const long long j_lo = ch * per, j_hi = min(nsamp, j_lo + per);
@@ -527,8 +518,8 @@ __global__ void __launch_bounds__(256) k_dw_moments(const __grid_constant__ DwPa
                     v = p.gscale[ax] * (p.recip[3 * ax] * p.disp[at] + p.recip[3 * ax + 1] * p.disp[at + 1] +
                                         p.recip[3 * ax + 2] * p.disp[at + 2]);
                 }
-                T q = k < n ? T(1) : T(0);
-                const T vt = (T)v;
+                CT q = k < n ? CT(1) : CT(0);
+                const CT vt = (CT)v;
                 for (int e = 0; e < P1; ++e) {
                     pw[(ax * P1 + e) * RS + k] = q;
                     q *= vt * inv_e[e];
@@ -538,9 +529,9 @@ __global__ void __launch_bounds__(256) k_dw_moments(const __grid_constant__ DwPa
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 if (ia[u] < 0) continue;
-                const T *x = pw + ia[u] * RS, *y = pw + (P1 + ib[u]) * RS, *z = pw + (2 * P1 + ic[u]) * RS;
+                const CT *x = pw + ia[u] * RS, *y = pw + (P1 + ib[u]) * RS, *z = pw + (2 * P1 + ic[u]) * RS;
                 for (int k0 = 0; k0 < DW_SUB; k0 += 16) {
-                    T t = T(0);
+                    CT t = CT(0);
 #pragma unroll
                     for (int k = 0; k < 16; ++k) t = fma(x[k0 + k] * y[k0 + k], z[k0 + k], t);
                     acc[u] += (double)t;
@@ -551,6 +542,20 @@ __global__ void __launch_bounds__(256) k_dw_moments(const __grid_constant__ DwPa
         for (int u = 0; u < 8; ++u)
             if (ia[u] >= 0) dst[dw_t0(P, ia[u], ib[u]) + ic[u]] = acc[u];
     }
+}
+template <typename T>
+__global__ void __launch_bounds__(256) k_dw_moments(const __grid_constant__ DwParams<T> p) {
+    __shared__ DwRoute rt;
+    __shared__ double inv_e[DW_PCAP + 1];           // 1 / (e + 1)
+    if (threadIdx.x == 0) {
+        rt = dw_route(p.xc, dw_eps<T>(), p.npts);
+        if (blockIdx.x == 0 && blockIdx.y == 0) p.route[0] = rt.P, p.route[1] = rt.taylor, p.route[2] = rt.wide;
+    }
+    __syncthreads();
+    if (!rt.taylor) return;
+    extern __shared__ __align__(16) unsigned char dw_raw[];
+    if (sizeof(T) == 8 || rt.wide) dw_moments_body<T, double>(p, rt.P, (double *)dw_raw, inv_e);
+    else dw_moments_body<T, T>(p, rt.P, (T *)dw_raw, (T *)inv_e);
 }
 
 // mom[site][t] = (-1)^(n/2) mean of the monomial (chunks added in order; odd orders 0)
@@ -919,8 +924,8 @@ void debye_waller_grid(const ds_model *M, const int g0[3], const int cnt[3], T *
         d.xc = xc;
         d.mom = mom;
         d.part = part;
-        const size_t sm = sizeof(T) * 3 * (DW_PCAP + 1) * (DW_SUB + 1);
-        if (sm > 48 * 1024) cudaFuncSetAttribute(k_dw_moments<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        constexpr size_t sm = sizeof(double) * 3 * (DW_PCAP + 1) * (DW_SUB + 1);   // the FP64 form's; FP32 takes half
+        static_assert(sm + 1024 <= 48 * 1024, "within the default shared memory of a block");
         k_dw_moments<T><<<dim3((unsigned)d.nchunk, (unsigned)d.nsite), 256, sm, st>>>(d);
         k_dw_reduce<T><<<dim3(8, (unsigned)d.nsite), 256, 0, st>>>(d);
         const size_t se = sizeof(double) * (DW_PCAP + 1) * (DW_PCAP + 1 + DW_ROWS);

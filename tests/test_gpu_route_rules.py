@@ -48,3 +48,22 @@ def test_debye_waller_grid_below_and_above_the_order_cap(ctx, spread, xmax):
     for prec, tag in PREC:
         got, _ = lm.intensity(qgrid_tuple(m.qgrid), disorder=1, mode=0, precision=prec, dw_coupling=1)
         assert np.max(np.abs(got.reshape(-1) - want)) / scale < TOL[tag], tag
+
+
+@pytest.mark.parametrize("xmax", [2.1, 4.0, 6.5])
+def test_debye_waller_moments_of_large_arguments_keep_fp32(ctx, xmax):
+    """Equal spins on atoms at +u or -u: each Bragg intensity is its value at rest times cos^2(Q.u), which the
+    polynomial forms from terms up to cosh(6.5) = 330 times as large.  With FP64 moments T_mu is right to
+    an FP32 rounding; the FP32 transform of 64 equal moments (6 stages), phase, |F|^2 and the projection
+    leave a few dozen roundings of 6e-8: 4e-6 of the peak."""
+    m = syn.small_case(syn.SPIN, cells=(4, 4, 4), nsite=1, nmodels=1, seed=244)
+    m.lattice = (4.0, 4.0, 4.0, 90.0, 90.0, 90.0)
+    m.spins = (np.zeros_like(m.spins) + np.array([0.6, -0.8, 0.0])).astype(np.float32)
+    m.qgrid = syn.QGrid(h0=(-2.0,) * 3, step=(0.25,) * 3, count=(17,) * 3)
+    u = np.array([1.0, 0.7, -0.4]) * np.random.default_rng(33).choice([-1.0, 1.0], m.spins.shape[:-1])[..., None]
+    m.disp = u.astype(np.float32)
+    m.disp = (u * (xmax / core.x_max(m, m.qgrid))).astype(np.float32)
+    G = m.qgrid.g_index(m.cells)
+    want = core.magnetic_intensity_fft(m, G, 0, dw=True)
+    got, _ = to_library(ctx, m).intensity(qgrid_tuple(m.qgrid), disorder=1, mode=0, precision=1, dw_coupling=1)
+    assert np.max(np.abs(got.reshape(-1) - want)) / np.max(core.magnetic_intensity_fft(m, G, 0)) < 4e-6
