@@ -763,7 +763,7 @@ ds_status queue_corner_xmax(ds_model *M, const ds_qgrid *q, const ds_opts *o, cu
     double *d_x = (double *)ws.get(sizeof(double) * 9);
     if (ws.failed) return ds_fail(ctx, DS_ERR_OOM, "device allocation failed");
     const size_t natom = (size_t)M->nmodels * M->nsite * M->n[0] * M->n[1] * M->n[2];
-    corner_xmax((int)natom, M->d_disp, corners, d_x, st);
+    corner_xmax((long long)natom, M->d_disp, corners, d_x, st);
     CK(cudaMemcpyAsync(host_out, d_x, sizeof(double) * 9, cudaMemcpyDeviceToHost, st));
     return DS_OK;
 }

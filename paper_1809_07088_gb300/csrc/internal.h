@@ -217,7 +217,7 @@ struct Corners {
     double v[24];  // 8 Cartesian Q vectors
 };
 // out (device, 9 doubles): max_j |Q_c . u_j| for the 8 corners, then max_j |u_j|
-void corner_xmax(int natom, const float *disp, const Corners &corners, double *out, cudaStream_t s);
+void corner_xmax(long long natom, const float *disp, const Corners &corners, double *out, cudaStream_t s);
 template <typename T> void recombine_cm(const RecombParams<T> &p, cudaStream_t s);
 // recomb_res.cu: the residue-class kernel when p.dres is set; false when it does not apply
 template <typename T> bool recombine_cm_residues(const RecombParams<T> &p, cudaStream_t s);

@@ -139,13 +139,13 @@ void site_means_spin(int nmodels, int nsite, int ncell, const float *spins, doub
 // out[c] = max_j |Q_c . u_j| for the 8 corners of the Q box (non-negative doubles order like
 // their bit patterns, so an integer atomicMax is exact)
 // out[8] = max_j |u_j| as well
-__global__ void k_corner_xmax(int natom, const float *disp, const Corners cq, unsigned long long *out) {
+__global__ void k_corner_xmax(long long natom, const float *disp, const Corners cq, unsigned long long *out) {
     const double *corners = cq.v;
     double best[9];
 #pragma unroll
     for (int c = 0; c < 9; ++c) best[c] = 0.0;
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < natom; j += gridDim.x * blockDim.x) {
-        const double ux = disp[3 * (size_t)j], uy = disp[3 * (size_t)j + 1], uz = disp[3 * (size_t)j + 2];
+    for (long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x; j < natom; j += gridDim.x * blockDim.x) {
+        const double ux = disp[3 * j], uy = disp[3 * j + 1], uz = disp[3 * j + 2];
 #pragma unroll
         for (int c = 0; c < 8; ++c)
             best[c] = fmax(best[c], fabs(corners[3 * c] * ux + corners[3 * c + 1] * uy + corners[3 * c + 2] * uz));
@@ -159,9 +159,9 @@ __global__ void k_corner_xmax(int natom, const float *disp, const Corners cq, un
     }
 }
 
-void corner_xmax(int natom, const float *disp, const Corners &corners, double *out, cudaStream_t s) {
+void corner_xmax(long long natom, const float *disp, const Corners &corners, double *out, cudaStream_t s) {
     cudaMemsetAsync(out, 0, 9 * sizeof(double), s);
-    int nb = std::min(1024, std::max(1, (natom + 255) / 256));
+    const int nb = (int)std::min<long long>(1024, std::max<long long>(1, (natom + 255) / 256));
     k_corner_xmax<<<nb, 256, 0, s>>>(natom, disp, corners, (unsigned long long *)out);
     count_launches(1);
 }

@@ -920,7 +920,7 @@ void debye_waller_grid(const ds_model *M, const int g0[3], const int cnt[3], T *
         d.route = route;
         Corners corners;
         box_corners(M, g0, cnt, corners.v);
-        corner_xmax((int)(nsamp * d.nsite), M->d_disp, corners, xc, st);
+        corner_xmax(nsamp * d.nsite, M->d_disp, corners, xc, st);
         d.xc = xc;
         d.mom = mom;
         d.part = part;
