@@ -819,7 +819,11 @@ size_t request_footprint(const ds_model *M, const ds_qgrid *q, const ds_opts *o,
         bytes += nf * (disp_spec_site(g.ncell_h, 1, SPEC_KB) - g.ncell_h) * ce;
     const int hl = lanczos_like(o) ? lanczos_halo(o->lanczos_m, o->lanczos_mprime) : 0;
     if (lanczos_like(o)) bytes += 3 * (cnt[0] + 2 * hl) * (cnt[1] + 2 * hl) * (cnt[2] + 2 * hl) * es;
-    if (o->dw_coupling) bytes += nsite * (cnt[0] + 2 * hl) * (cnt[1] + 2 * hl) * (cnt[2] + 2 * hl) * es;
+    if (o->dw_coupling) {
+        bytes += nsite * (cnt[0] + 2 * hl) * (cnt[1] + 2 * hl) * (cnt[2] + 2 * hl) * es;
+        const size_t moments = debye_waller_scratch(M);   // left out by the request where it does not fit
+        if (bytes + moments <= M->ctx->budget) bytes += moments;
+    }
     return bytes;
 }
 

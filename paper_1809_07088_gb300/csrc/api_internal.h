@@ -173,6 +173,8 @@ bool lanczos_like(const ds_opts *o);
 double sphere_cutoff_radius(const ds_model *M, int m, int mprime);
 double sphere_profile(double x);
 void sphere_stencil_weights(const ds_model *M, int m, int mprime, int h, std::vector<double> &w);
+// scratch of the moment route of T_mu(G) (subbox_dft.cu), taken where it fits the budget
+size_t debye_waller_scratch(const ds_model *M);
 // T_mu(G) of Eq. dw on the grid g0 + [0, cnt) of supercell indices, [site][voxel] (subbox_dft.cu)
 template <typename T>
 void debye_waller_grid(const ds_model *M, const int g0[3], const int cnt[3], T *out, Scratch &ws, cudaStream_t st);

@@ -893,6 +893,15 @@ ds_status run_debye_waller(ds_model *Mdl, const double *hkl, long long npts, int
 
 }  // namespace
 
+// chunks of the moment sums: at least 256 lattice points each, about two CTAs per SM over the sites
+static int dw_chunks(const ds_model *M) {
+    const long long nsamp = (long long)M->nmodels * M->n[0] * M->n[1] * M->n[2];
+    return (int)std::max<long long>(1, std::min<long long>((nsamp + 255) / 256, (152 * 2 + M->nsite - 1) / M->nsite));
+}
+size_t debye_waller_scratch(const ds_model *M) {
+    return sizeof(double) * (12 + (size_t)DW_T * M->nsite * (1 + (size_t)dw_chunks(M)));
+}
+
 // T_mu(G) on the computing grid of a magnetic request, [site][voxel] (api.cu)
 template <typename T>
 void debye_waller_grid(const ds_model *M, const int g0[3], const int cnt[3], T *out, Scratch &ws, cudaStream_t st) {
@@ -910,20 +919,18 @@ void debye_waller_grid(const ds_model *M, const int g0[3], const int cnt[3], T *
     d.pt_stride = 1;
     d.out = out;
     const long long nsamp = (long long)d.nmodels * d.ncell;
-    // moment route: chunks of at least 256 lattice points, about two CTAs per SM over the sites
-    d.nchunk = (int)std::max<long long>(1, std::min<long long>((nsamp + 255) / 256, (152 * 2 + d.nsite - 1) / d.nsite));
-    double *xc = (double *)ws.get(sizeof(double) * 9);
-    double *mom = (double *)ws.get(sizeof(double) * DW_T * d.nsite);
-    double *part = (double *)ws.get(sizeof(double) * DW_T * d.nsite * (size_t)d.nchunk);
-    int *route = (int *)ws.get(sizeof(int) * 3);
-    if (!ws.failed) {
-        d.route = route;
+    d.nchunk = dw_chunks(M);
+    // one block, so that nothing is held when it does not fit: corner maxima, route, moments, their chunks
+    const size_t need = debye_waller_scratch(M);
+    double *block = ws.total + need <= M->ctx->budget ? (double *)ws.get(need) : nullptr;
+    if (block) {
+        d.xc = block;
+        d.route = (int *)(block + 10);
+        d.mom = block + 12;
+        d.part = d.mom + (size_t)DW_T * d.nsite;
         Corners corners;
         box_corners(M, g0, cnt, corners.v);
-        corner_xmax(nsamp * d.nsite, M->d_disp, corners, xc, st);
-        d.xc = xc;
-        d.mom = mom;
-        d.part = part;
+        corner_xmax(nsamp * d.nsite, M->d_disp, corners, block, st);
         constexpr size_t sm = sizeof(double) * 3 * (DW_PCAP + 1) * (DW_SUB + 1);   // the FP64 form's; FP32 takes half
         static_assert(sm + 1024 <= 48 * 1024, "within the default shared memory of a block");
         k_dw_moments<T><<<dim3((unsigned)d.nchunk, (unsigned)d.nsite), 256, sm, st>>>(d);
@@ -932,7 +939,7 @@ void debye_waller_grid(const ds_model *M, const int g0[3], const int cnt[3], T *
         k_dw_eval<T><<<dim3((unsigned)cnt[0], (unsigned)d.nsite), DW_ETHR, se, st>>>(d);
         count_launches(3);
     } else {
-        ws.failed = false;   // no scratch for the moments: the direct sum needs none
+        ws.failed = false;   // no memory for the moments: the direct sum needs none
     }
     constexpr int VPT = 8;
     const long long nwork = (long long)cnt[0] * cnt[1] * ((cnt[2] + VPT - 1) / VPT);

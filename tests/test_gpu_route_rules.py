@@ -67,3 +67,23 @@ def test_debye_waller_moments_of_large_arguments_keep_fp32(ctx, xmax):
     want = core.magnetic_intensity_fft(m, G, 0, dw=True)
     got, _ = to_library(ctx, m).intensity(qgrid_tuple(m.qgrid), disorder=1, mode=0, precision=1, dw_coupling=1)
     assert np.max(np.abs(got.reshape(-1) - want)) / np.max(core.magnetic_intensity_fft(m, G, 0)) < 4e-6
+
+
+@pytest.mark.parametrize("prec,tag", PREC)
+def test_debye_waller_moments_stay_within_the_budget(ctx, prec, tag):
+    """The scratch of the moments counts against the context's budget: with one byte too little for it the
+    direct sum, which needs none, serves the request."""
+    import paper_1809_07088_gb300 as ds
+    m = _dw_model("gauss", 1.0)
+    G = m.qgrid.g_index(m.cells)
+    want = core.magnetic_intensity_fft(m, G, 0, dw=True)
+    scale = np.max(core.magnetic_intensity_fft(m, G, 0))
+    opts = dict(disorder=1, mode=0, precision=prec, dw_coupling=1)
+    _, info = to_library(ctx, m).intensity(qgrid_tuple(m.qgrid), **opts)
+    small = ds.Context(0, info["workspace_bytes"] - 1)
+    try:
+        got, info2 = to_library(small, m).intensity(qgrid_tuple(m.qgrid), **opts)
+    finally:
+        small.close()
+    assert info2["workspace_bytes"] < info["workspace_bytes"]
+    assert np.max(np.abs(got.reshape(-1) - want)) / scale < TOL[tag]
