@@ -50,10 +50,11 @@ template <typename T> struct SxParams {
     int nq, ld;                     // points of the chunk, and padded to whole blocks
     long long ldp;                  // stride of the constants
     double recip[9];
-    c_t<T> *phi;                    // [site][ldp]: phi_mu; displacements (b f, Q.r_mu in cycles)
+    c_t<T> *phi;                    // [site][ldp]: phi_mu
     c_t<T> *e;                      // [axis][ldp]
     T *Q;                           // [axis][ldp]: Q / 2 pi (cycles per A) for displacements, Q for moments
-    c_t<T> *B, *K;                  // displacements: box sum of exp(2 pi i Q.d); others: mean amplitude [comp][ldp]
+    double2 *phiB;                  // displacements: [site][ldp]: phi_mu times the box sum of exp(2 pi i Q.d)
+    c_t<T> *K;                      // occupancies, moments: mean amplitude [comp][ldp]
     c_t<T> *A, *L;                  // [comp][model cell][ld]; A: amplitudes where the line sums take their own pass
     T *dwp, *dwm;                   // [row block][site][ld]: sums of w cos(Q.u); [site][ld]: their mean
     int rows_per, nrb;              // rows of cells per block, row blocks
@@ -75,33 +76,6 @@ template <typename T, int KIND> __global__ void __launch_bounds__(SX_T) k_sx_pre
         p.Q[a * p.ldp + j] = (T)(KIND == SB_DISP ? Qd[a] / TWO_PI_D : Qd[a]);
     }
     const double s2 = (Qd[0] * Qd[0] + Qd[1] * Qd[1] + Qd[2] * Qd[2]) / (FOUR_PI_D * FOUR_PI_D);
-    constexpr int NC = KIND == SB_SPIN ? 3 : 1;
-    double Kr[NC], Ki[NC];
-#pragma unroll
-    for (int c = 0; c < NC; ++c) Kr[c] = Ki[c] = 0.0;
-    for (int s = 0; s < p.nsite; ++s) {
-        const SbSite &S = p.site[s];
-        const double f = S.b * form_factor<double>(S.kind, S.coef, s2);
-        const double t = frac_w(h[0] * S.r[0] + h[1] * S.r[1] + h[2] * S.r[2]);
-        if (KIND == SB_DISP) {
-            p.phi[s * p.ldp + j] = mk<T>((T)f, (T)t);
-            continue;
-        }
-        double sn, cs;
-        sincospi(2.0 * t, &sn, &cs);
-        p.phi[s * p.ldp + j] = mk<T>((T)(f * cs), (T)(f * sn));
-        if (p.diffuse) {
-#pragma unroll
-            for (int c = 0; c < NC; ++c) {
-                const double m = p.mean[KIND == SB_SPIN ? 3 * s + c : s];
-                Kr[c] += f * cs * m;
-                Ki[c] += f * sn * m;
-            }
-        }
-    }
-    if (KIND != SB_DISP)
-#pragma unroll
-        for (int c = 0; c < NC; ++c) p.K[c * p.ldp + j] = mk<T>((T)Kr[c], (T)Ki[c]);
     double Br = 1.0, Bi = 0.0;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -120,7 +94,30 @@ template <typename T, int KIND> __global__ void __launch_bounds__(SX_T) k_sx_pre
         Bi = Br * si + Bi * sr;
         Br = t;
     }
-    if (KIND == SB_DISP) p.B[j] = mk<T>((T)Br, (T)Bi);
+    constexpr int NC = KIND == SB_SPIN ? 3 : 1;
+    double Kr[NC], Ki[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) Kr[c] = Ki[c] = 0.0;
+    for (int s = 0; s < p.nsite; ++s) {
+        const SbSite &S = p.site[s];
+        const double f = S.b * form_factor<double>(S.kind, S.coef, s2);
+        const double t = frac_w(h[0] * S.r[0] + h[1] * S.r[1] + h[2] * S.r[2]);
+        double sn, cs;
+        sincospi(2.0 * t, &sn, &cs);
+        p.phi[s * p.ldp + j] = mk<T>((T)(f * cs), (T)(f * sn));
+        if (KIND == SB_DISP && p.diffuse) p.phiB[s * p.ldp + j] = make_double2(f * cs * Br - f * sn * Bi, f * cs * Bi + f * sn * Br);
+        if (KIND != SB_DISP && p.diffuse) {
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                const double m = p.mean[KIND == SB_SPIN ? 3 * s + c : s];
+                Kr[c] += f * cs * m;
+                Ki[c] += f * sn * m;
+            }
+        }
+    }
+    if (KIND != SB_DISP)
+#pragma unroll
+        for (int c = 0; c < NC; ++c) p.K[c * p.ldp + j] = mk<T>((T)Kr[c], (T)Ki[c]);
 }
 
 // x e + a for complex x, e, a
@@ -132,9 +129,9 @@ template <typename C> __device__ __forceinline__ C cmad(C x, C e, C a) {
 }
 
 // Line sums (LINE) or plain amplitudes of whole rows of cells.  The row loop is unrolled by the ring
-// length, so the ring is indexed by constants.  Displacements: the site phase Q.r_mu is added to each
-// atom's phase, so an atom costs three multiply-adds, one reduction, one (sin, cos) pair and two
-// multiply-adds; the sums of its (cos, sin) per site give the Debye-Waller mean.  Sites beyond nsite
+// length, so the ring is indexed by constants.  Displacements: an atom costs three multiply-adds, one
+// reduction, one (sin, cos) pair, the product with its site's factor (four multiply-adds; formed in FP64
+// and rounded once, as box by box) and one add into its site's sum of cosines, the Debye-Waller mean.  Sites beyond nsite
 // (MAXS > nsite) are atoms of weight zero.  WGT: occupancies weight the displaced atoms.
 template <typename T, int KIND, int MAXS, bool LINE, bool WGT>
 __global__ void __launch_bounds__(SX_T, sizeof(T) == 4 && MAXS <= 4 && KIND != SB_SPIN ? 8 : 4) k_sx_rows(const __grid_constant__ SxParams<T> p) {
@@ -146,11 +143,12 @@ __global__ void __launch_bounds__(SX_T, sizeof(T) == 4 && MAXS <= 4 && KIND != S
     C *first = (C *)(sx_raw + sizeof(float4) * n3 * MAXS) + tid;   // LINE: [i][comp][SX_T], a row's first amplitudes
     const int ql = blockIdx.x * SX_T + tid;
     const long long j = p.q0 + ql;                     // < ldp: chunks are whole blocks
-    C phi[MAXS], wsum[KIND == SB_DISP ? MAXS : 1];
+    C phi[MAXS];
+    T wsum[KIND == SB_DISP ? MAXS : 1];
 #pragma unroll
     for (int s = 0; s < MAXS; ++s) {
         phi[s] = s < nsite ? p.phi[s * p.ldp + j] : mk<T>(T(0), T(0));
-        if (KIND == SB_DISP) wsum[KIND == SB_DISP ? s : 0] = mk<T>(T(0), T(0));
+        if (KIND == SB_DISP) wsum[KIND == SB_DISP ? s : 0] = T(0);
     }
     const C e3 = p.e[2 * p.ldp + j];
     T Qx = T(0), Qy = T(0), Qz = T(0);
@@ -197,18 +195,15 @@ __global__ void __launch_bounds__(SX_T, sizeof(T) == 4 && MAXS <= 4 && KIND != S
 #pragma unroll
                         for (int s = 0; s < MAXS; ++s) {
                             const float4 v = at[s];
-                            const T t = fma(Qx, (T)v.x, fma(Qy, (T)v.y, fma(Qz, (T)v.z, phi[s].y)));
+                            const T t = fma(Qx, (T)v.x, fma(Qy, (T)v.y, Qz * (T)v.z));
                             T cs, sn;
                             sincos_cycles(frac_w(t), cs, sn);
                             if (WGT) {
                                 cs *= (T)v.w;
                                 sn *= (T)v.w;
                             }
-                            C &ws = wsum[KIND == SB_DISP ? s : 0];
-                            ws.x += cs;
-                            ws.y += sn;
-                            a[0].x = fma(phi[s].x, cs, a[0].x);
-                            a[0].y = fma(phi[s].x, sn, a[0].y);
+                            wsum[KIND == SB_DISP ? s : 0] += cs;
+                            a[0] = cmad(phi[s], mk<T>(cs, sn), a[0]);
                         }
                     } else {
 #pragma unroll
@@ -258,15 +253,9 @@ __global__ void __launch_bounds__(SX_T, sizeof(T) == 4 && MAXS <= 4 && KIND != S
         }
     }
     if (KIND == SB_DISP && p.diffuse) {
-        // sum of w cos(Q.u) = Re[exp(-iQ.r_mu) sum of w exp(i(Q.u + Q.r_mu))]
 #pragma unroll
         for (int s = 0; s < MAXS; ++s)
-            if (s < nsite) {
-                T cs, sn;
-                sincos_cycles(phi[s].y, cs, sn);
-                const C ws = wsum[KIND == SB_DISP ? s : 0];
-                p.dwp[((size_t)blockIdx.y * nsite + s) * p.ld + ql] = fma(ws.x, cs, ws.y * sn);
-            }
+            if (s < nsite) p.dwp[((size_t)blockIdx.y * nsite + s) * p.ld + ql] = wsum[KIND == SB_DISP ? s : 0];
     }
 }
 
@@ -341,17 +330,15 @@ __global__ void __launch_bounds__(SX_T) k_sx_boxes(const __grid_constant__ SxPar
     const C e2n = cmul(pw[NB - 1], e2);
     C KB = mk<T>(T(0), T(0));
     if (KIND == SB_DISP && p.diffuse) {
-        // K B, K = sum_mu phi_mu <w cos(Q.u)>_mu
-        C k = mk<T>(T(0), T(0));
+        // K B, K = sum_mu phi_mu <w cos(Q.u)>_mu: cancels against F at Bragg positions, so FP64, rounded once
+        double kr = 0.0, ki = 0.0;
         for (int s = 0; s < p.nsite; ++s) {
-            const C ph = p.phi[s * p.ldp + j];
-            T cs, sn;
-            sincos_cycles(ph.y, cs, sn);
-            const T f = ph.x * p.dwm[(size_t)s * p.ld + ql];
-            k.x = fma(f, cs, k.x);
-            k.y = fma(f, sn, k.y);
+            const double2 pb = p.phiB[s * p.ldp + j];
+            const double w = (double)p.dwm[(size_t)s * p.ld + ql];
+            kr = fma(pb.x, w, kr);
+            ki = fma(pb.y, w, ki);
         }
-        KB = cmul(k, p.B[j]);
+        KB = mk<T>((T)kr, (T)ki);
     }
     T Qv[3] = {T(0), T(0), T(0)};
     if (KIND == SB_SPIN)
@@ -552,18 +539,20 @@ bool subbox_cells_run(ds_model *M, int kind, const SbSite *d_sites, const int4 *
     if ((norigin + p.per_chunk - 1) / p.per_chunk > 65535) return false;
     const int nochunk = (int)((norigin + p.per_chunk - 1) / p.per_chunk);
     const size_t nk = (size_t)p.ldp, before = ws.total;
-    const size_t need = sizeof(C) * nk * (nsite + 3 + 1 + NC) + sizeof(T) * 3 * nk + (size_t)chunk_q * per_q +
-                        (kind == SB_DISP && p.diffuse ? sizeof(T) * (size_t)(p.nrb + 1) * nsite * p.ld : 0) +
+    const bool mean_b = kind == SB_DISP && p.diffuse;
+    const size_t need = sizeof(C) * nk * (nsite + 3 + NC) + sizeof(T) * 3 * nk + (size_t)chunk_q * per_q +
+                        (mean_b ? sizeof(double2) * nk * nsite : 0) +
+                        (mean_b ? sizeof(T) * (size_t)(p.nrb + 1) * nsite * p.ld : 0) +
                         sizeof(T) * (size_t)nochunk * npts;
     if (before + need > ctx->budget) return false;
     p.phi = (C *)ws.get(sizeof(C) * nk * nsite);
     p.e = (C *)ws.get(sizeof(C) * nk * 3);
     p.Q = (T *)ws.get(sizeof(T) * nk * 3);
-    p.B = (C *)ws.get(sizeof(C) * nk);
+    if (mean_b) p.phiB = (double2 *)ws.get(sizeof(double2) * nk * nsite);
     p.K = (C *)ws.get(sizeof(C) * nk * NC);
     p.L = (C *)ws.get(sizeof(C) * (size_t)cells * NC * p.ld);
     if (nsb > SX_RING) p.A = (C *)ws.get(sizeof(C) * (size_t)cells * NC * p.ld);
-    if (kind == SB_DISP && p.diffuse) {
+    if (mean_b) {
         p.dwp = (T *)ws.get(sizeof(T) * (size_t)(p.nrb + 1) * nsite * p.ld);
         p.dwm = p.dwp + (size_t)p.nrb * nsite * p.ld;
     }

@@ -87,3 +87,41 @@ def test_debye_waller_moments_stay_within_the_budget(ctx, prec, tag):
         small.close()
     assert info2["workspace_bytes"] < info["workspace_bytes"]
     assert np.max(np.abs(got.reshape(-1) - want)) / scale < TOL[tag]
+
+
+def _undisplaced(sites):
+    m = syn.small_case(syn.DISP, cells=(6, 5, 4), nsite=len(sites), nmodels=1, seed=242)
+    m.sites = np.array(sites, dtype=np.float64)
+    m.scat_len = np.full(len(sites), 1.3)
+    m.ff_kind = np.zeros(len(sites), np.int32)
+    m.ff_coef = np.zeros((len(sites), 9))
+    m.occ = None
+    m.disp = np.zeros_like(m.disp)
+    return m
+
+
+@pytest.mark.parametrize("nsb", [3, 4])
+def test_subbox_points_systematic_absences_are_zero(ctx, nsb):
+    """Three equal sites a third of a cell apart cancel exactly in FP32 at h not divisible by three when the
+    atoms are not displaced: their factors 1, -1/2 + is and -1/2 - is are formed in FP64 and rounded
+    once, and every other factor is shared by overlapping boxes."""
+    m = _undisplaced([[0.0, 0.0, 0.0], [1.0 / 3.0, 0.0, 0.0], [2.0 / 3.0, 0.0, 0.0]])
+    m.scat_len = np.ones(3)
+    rng = np.random.default_rng(31)
+    hkl = np.stack([rng.choice([-5.0, -2.0, -1.0, 1.0, 2.0, 4.0], 200), *rng.uniform(-2.0, 2.0, (2, 200))], -1)
+    org = syn.random_origins(rng, 1, m.cells, 360)
+    got, _ = to_library(ctx, m).subbox_points(hkl, org, disorder=2, mode=0, precision=1, subbox_n=nsb)
+    assert np.all(got == 0.0)
+
+
+@pytest.mark.parametrize("prec,tag", PREC)
+def test_subbox_points_mean_term_of_an_undisplaced_crystal(ctx, prec, tag):
+    """DIFFUSE boxes of an undisplaced crystal at Bragg positions: <cos(Q.u)> = 1, the box phases are 1 and
+    2^3 cells add without rounding, so F = 8 phi and the mean term, formed in FP64 and rounded once, is
+    the same number."""
+    m = _undisplaced([[0.3, 0.17, 0.71]])
+    rng = np.random.default_rng(32)
+    hkl = rng.integers(-6, 7, (200, 3)).astype(np.float64)
+    org = syn.random_origins(rng, 1, m.cells, 360)
+    got, _ = to_library(ctx, m).subbox_points(hkl, org, disorder=2, mode=1, precision=prec, subbox_n=2)
+    assert np.all(got == 0.0)
