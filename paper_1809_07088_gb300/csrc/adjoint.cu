@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(fi_threads<N>(), 1)
 template <typename T, int N>
 void launch_field_inv(const c_t<T> *in, size_t nf, T *out, const int4 *terms, int nT, cudaStream_t s) {
     constexpr size_t sm = (size_t)N * N * (N / 2 + 1) * sizeof(c_t<T>);
-    if (sm > 48 * 1024) cudaFuncSetAttribute(k_fft_field_inv<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    allow_smem(k_fft_field_inv<T, N>, sm);
     k_fft_field_inv<T, N><<<(unsigned)nf, fi_threads<N>(), sm, s>>>(in, 0, out, terms, nT);
     count_launches(1);
 }
@@ -255,8 +255,7 @@ void fft_complex_realpart(const Geometry &g, const c_t<T> *in, int f0, int nf, c
         }
     }
     const size_t sm1 = (g.n[1] + g.n[2] + 2 * (size_t)g.n[1] * g.n[2]) * sizeof(C);
-    if (sm1 > 48 * 1024)
-        cudaFuncSetAttribute(k_fft_planes_c<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1);
+    allow_smem(k_fft_planes_c<T>, sm1);
     k_fft_planes_c<T><<<(unsigned)((size_t)g.n[0] * nf), 256, sm1, s>>>(g, in, f0, work, W[1], W[2]);
     const int ncol = g.n[1] * g.n[2];
     int cb = (int)((48 * 1024 / sizeof(C) - g.n[0]) / (2 * g.n[0]));
@@ -592,7 +591,7 @@ ds_status backward_run(ds_model *M, const ds_qgrid *q, const ds_opts *o, const T
                 constexpr int TPT = sizeof(T) == 4 ? 4 : 2;
                 const size_t sm = (size_t)ADJ_ZC * nsite * sizeof(C) + (size_t)ADJ_ZC * 3 * (keep.src.P + 1) * sizeof(T);
                 auto launch = [&](auto kern, int tpt) {
-                    if (sm > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+                    allow_smem(kern, sm);
                     dim3 gr(g.ncell, (nT + 256 * tpt - 1) / (256 * tpt));
                     kern<<<gr, 256, sm, st>>>(p, dLdI, F, keep.src.P, 2.0 / (nmod * N), Z);
                 };
@@ -638,7 +637,7 @@ ds_status backward_run(ds_model *M, const ds_qgrid *q, const ds_opts *o, const T
                 for (int a = 0; a < 3; ++a) ax.bg[3 * j + a] = p.gscale[j] * p.recip[3 * j + a];
             const int P = keep.src.P;
             const size_t sm = sizeof(T) * AG_CELLS * (P + 1 + 3 * AG_SLICES);
-            if (sm > 48 * 1024) cudaFuncSetAttribute(k_adj_gather<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+            allow_smem(k_adj_gather<T>, sm);
             // (model, site) pairs on the grid's y axis, at most 65535 per launch
             for (int ms0 = 0; ms0 < nmod * nsite; ms0 += 65535) {
                 const int nms = std::min(65535, nmod * nsite - ms0);

@@ -258,15 +258,15 @@ bool adjoint_z_disp_sf(const RecombParams<float> &p, const float *dLdI, const fl
     const unsigned nb = (unsigned)(half ? p.g.ncell_h : p.g.ncell);
     switch (sf_threads_for(L.total)) {
         case 128:
-            cudaFuncSetAttribute(k_adj_taylor_sf<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total);
+            allow_smem(k_adj_taylor_sf<128>, L.total);
             k_adj_taylor_sf<128><<<nb, 128, L.total, s>>>(p, dLdI, F, P, zr, (float)scale, half ? 1 : 0, Z);
             break;
         case 256:
-            cudaFuncSetAttribute(k_adj_taylor_sf<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total);
+            allow_smem(k_adj_taylor_sf<256>, L.total);
             k_adj_taylor_sf<256><<<nb, 256, L.total, s>>>(p, dLdI, F, P, zr, (float)scale, half ? 1 : 0, Z);
             break;
         default:
-            cudaFuncSetAttribute(k_adj_taylor_sf<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total);
+            allow_smem(k_adj_taylor_sf<512>, L.total);
             k_adj_taylor_sf<512><<<nb, 512, L.total, s>>>(p, dLdI, F, P, zr, (float)scale, half ? 1 : 0, Z);
             break;
     }

@@ -387,8 +387,7 @@ __global__ void __launch_bounds__(fr_threads<N1>(), 1) k_fft_field_reg(const Geo
 template <typename T, int N> static bool launch_field_reg(const Geometry &g, const FieldSource &src, int f0, int nf,
                                                           c_t<T> *spec, cudaStream_t s) {
     constexpr size_t sm = (size_t)N * N * (N / 2 + 1) * sizeof(c_t<T>);
-    if (sm > 48 * 1024)
-        cudaFuncSetAttribute(k_fft_field_reg<T, N, N, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    allow_smem(k_fft_field_reg<T, N, N, N>, sm);
     k_fft_field_reg<T, N, N, N><<<(unsigned)nf, fr_threads<N>(), sm, s>>>(g, src, f0, spec);
     count_launches(1);
     return true;
@@ -668,7 +667,7 @@ static void fft_two_pass(const Geometry &g, const FieldSource &src, int f0, int 
     const int n2p = (g.n[1] + 1) / 2;
     const size_t plane_c = (size_t)std::max(n2p * g.n[2], g.n[1] * g.n3h);
     size_t sm1 = (g.n[1] + g.n[2] + 2 * ppc * plane_c) * ce;
-    if (sm1 > 48 * 1024) cudaFuncSetAttribute(k_fft_planes<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1);
+    allow_smem(k_fft_planes<T>, sm1);
     dim3 g1((unsigned)(((g.n[0] + ppc - 1) / ppc) * (size_t)nf));
     k_fft_planes<T><<<g1, 256, sm1, s>>>(g, src, f0, ppc, work, W2, W3);
     // pass 2
@@ -693,7 +692,7 @@ void fft_real_fields(const Geometry &g, const FieldSource &src, int f0, int nf, 
     // supercells of at least 18^3 cells (measured on GB300: 1.4x faster than the two passes at
     // 20^3 x 1024 fields, even at 16^3 x 2000, slower for 8^3 or for fewer fields)
     if (const size_t smf = (nf >= 4 * 152 && g.ncell >= 5832) ? field_smem(g, sizeof(c_t<T>)) : 0) {
-        if (smf > 48 * 1024) cudaFuncSetAttribute(k_fft_field<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smf);
+        allow_smem(k_fft_field<T>, smf);
         k_fft_field<T><<<(unsigned)nf, 512, smf, s>>>(g, src, f0, spec, W1, W2, W3);
         count_launches(1);
         return;

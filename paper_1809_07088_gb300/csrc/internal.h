@@ -196,6 +196,17 @@ template <typename T> inline void set_reciprocal(RecombParams<T> &p, const doubl
     }
 }
 
+// A kernel's limit of dynamic shared memory is state of the device, shared by every thread that launches it
+// (callers, the serving worker).  It is raised to all that a block may have beside the kernel's static
+// part, whatever this launch needs, so that no request lowers it between another's call here and its
+// launch.  Launches within the default limit leave it alone.
+template <typename K> inline void allow_smem(K kern, size_t bytes) {
+    if (bytes <= 40 * 1024) return;   // the default, 48 KB, holds the static part too
+    cudaFuncAttributes a;
+    if (cudaFuncGetAttributes(&a, kern) != cudaSuccess) return;   // the launch reports it
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - (int)a.sharedSizeBytes);
+}
+
 // ---- launchers (fft.cu) --------------------------------------------------------------------
 template <typename T> void make_twiddles(int n, c_t<T> *W, cudaStream_t s);
 template <typename T>

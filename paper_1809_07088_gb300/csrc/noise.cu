@@ -275,7 +275,7 @@ static void sliding_passes(const T *ext, T *tmp1, T *tmp2, T *out, int d[3], con
         const int L = run_len(nseg, d[0], Bo);
         const int nrun = (Bo + L - 1) / L;
         const size_t sm = (size_t)plane_depth<NT>() * plane_slot<T, NT>(nthr) * sizeof(T);
-        if (sm > 48 * 1024) cudaFuncSetAttribute(k_lanczos_plane<T, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        allow_smem(k_lanczos_plane<T, NT>, sm);
         dim3 grid((unsigned)((Co + 2 * nthr - 1) / (2 * nthr)), (unsigned)(d[0] * nrun));
         k_lanczos_plane<T, NT><<<grid, nthr, sm, s>>>(ext, tmp1, d[0], d[1], d[2], L, tp);
         d[1] = Bo;
@@ -361,7 +361,7 @@ void sphere_resample(const T *ext, const T *w, T *out, const int cnt[3], int h, 
     const size_t tot = (size_t)cnt[0] * cnt[1] * cnt[2];
     const int nt = 2 * h + 1;
     const size_t sm = (size_t)nt * nt * nt * sizeof(T);
-    if (sm > 48 * 1024) cudaFuncSetAttribute(k_sphere_stencil<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    allow_smem(k_sphere_stencil<T>, sm);
     const unsigned nb = (unsigned)std::max<size_t>(1, std::min<size_t>((tot + 255) / 256, 152 * 16));
     k_sphere_stencil<T><<<nb, 256, sm, s>>>(ext, w, out, cnt[0], cnt[1], cnt[2], h);
     count_launches(1);

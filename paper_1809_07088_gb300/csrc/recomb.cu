@@ -383,9 +383,7 @@ void launch_cm_variant(const RecombParams<T> &p, int per, cudaStream_t s) {
     const int nH12 = p.gm.nH[0] * p.gm.nH[1];
     const int ktiles = (p.g.ncell + 255) / 256;
     const size_t sm = (size_t)per * p.gm.nH[2] * p.nsite * sizeof(C);
-    if (sm > 48 * 1024)
-        cudaFuncSetAttribute(k_recomb_cm<T, NC, MAXS, ONECLS, VPI, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)sm);
+    allow_smem(k_recomb_cm<T, NC, MAXS, ONECLS, VPI, MINB>, sm);
     dim3 grid(ktiles, (nH12 + per - 1) / per);
     k_recomb_cm<T, NC, MAXS, ONECLS, VPI, MINB><<<grid, 256, sm, s>>>(p, per);
     count_launches(1);
@@ -612,9 +610,7 @@ void launch_cm_grp_variant(const RecombParams<T> &p, int per, cudaStream_t s) {
     const int ktiles = (p.g.ncell + 255) / 256;
     size_t sm = ((size_t)per * p.nsite + (size_t)(p.gm.nH[2] + 1) * p.grp.ngrp) * sizeof(C);
     if (YSMEM) sm += (size_t)p.nsite * NC * 256 * sizeof(C);
-    if (sm > 48 * 1024)
-        cudaFuncSetAttribute(k_recomb_cm_grp<T, NC, MAXS, MAXG, ONECLS, VPI, MINB, YSMEM>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    allow_smem(k_recomb_cm_grp<T, NC, MAXS, MAXG, ONECLS, VPI, MINB, YSMEM>, sm);
     dim3 grid(ktiles, (nH12 + per - 1) / per);
     k_recomb_cm_grp<T, NC, MAXS, MAXG, ONECLS, VPI, MINB, YSMEM><<<grid, 256, sm, s>>>(p, per);
     count_launches(1);
@@ -995,8 +991,7 @@ template <typename T, int NS, int ZPT, int MINB> static void launch_disp(const R
     for (int a = 0; a < 3; ++a) nzmax *= (p.gm.cnt[a] + p.g.n[a] - 1) / p.g.n[a] + 1;
     dim3 grid((p.g.ncell + DISP_KT - 1) / DISP_KT, (nzmax + 32 * ZPT - 1) / (32 * ZPT));
     const size_t sm = 2 * (size_t)DISP_KT * NS * DISP_TC * sizeof(C) + 2 * DISP_TC * sizeof(int);
-    if (sm > 48 * 1024)
-        cudaFuncSetAttribute(k_recomb_disp<T, NS, ZPT, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    allow_smem(k_recomb_disp<T, NS, ZPT, MINB>, sm);
     k_recomb_disp<T, NS, ZPT, MINB><<<grid, DISP_KT * 32, sm, s>>>(p);
     count_launches(1);
 }
@@ -1103,7 +1098,7 @@ void displacive_bragg(const RecombParams<T> &p, const int4 *terms, c_t<T> *avg0,
     int P = 0;   // the order of the nT monomials: (P + 1)(P + 2)(P + 3) / 6 = nT
     while ((P + 1) * (P + 2) * (P + 3) / 6 < p.nT) ++P;
     const size_t sm = (size_t)8 * 3 * (P + 1) * sizeof(double);
-    if (sm > 48 * 1024) cudaFuncSetAttribute(k_bragg_disp<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    allow_smem(k_bragg_disp<T>, sm);
     k_bragg_disp<T><<<(nz + 7) / 8, 256, sm, s>>>(p, avg0, bragg, P);
     count_launches(2);
 }

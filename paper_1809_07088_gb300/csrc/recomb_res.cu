@@ -277,9 +277,7 @@ static void launch_res(const RecombParams<T> &p, cudaStream_t s) {
     const int nchunk = (p.dres[2] + D3 - 1) / D3;
     const int s3 = res_split(ktiles * d12, nchunk, 152 * MINB, 1);
     const size_t sm = (size_t)p.dres[2] * p.nsite * sizeof(C);
-    if (sm > 48 * 1024)
-        cudaFuncSetAttribute(k_recomb_cm_res<T, NC, MAXC, D3, MINB, ACC, NG>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    allow_smem(k_recomb_cm_res<T, NC, MAXC, D3, MINB, ACC, NG>, sm);
     dim3 grid(ktiles, d12 * s3);
     k_recomb_cm_res<T, NC, MAXC, D3, MINB, ACC, NG><<<grid, RES_THREADS, sm, s>>>(p, s3);
     count_launches(1);

@@ -578,8 +578,7 @@ template <typename T, int NC, int NG, bool ORTHO, bool ACC> static void launch_r
     ax.dqm = ax.dq % p.dres[2];
     ax.symm = 1;
     for (int a = 0; a < 3; ++a) ax.symm &= 2 * p.gm.g0[a] + p.gm.cnt[a] == 1;
-    if (L.total > 48 * 1024)
-        cudaFuncSetAttribute(k_recomb_rows<T, NC, NG, ORTHO, ACC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total);
+    allow_smem(k_recomb_rows<T, NC, NG, ORTHO, ACC>, L.total);
     // programmatic dependent launch: the CTAs may start (decoding, zone phases) while the
     // transform before them in the stream finishes; they wait for it before reading its output
     cudaLaunchConfig_t cfg = {};

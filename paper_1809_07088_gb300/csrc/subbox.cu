@@ -186,8 +186,7 @@ bool corr_planes(const Geometry &g, int nmodels, int nfield, int npair, const in
         if (2 * nsb - 1 != W) return corr_planes<T, W + 2>(g, nmodels, nfield, npair, pairs, x, nsb, wc, st);
         const CorrLayout L = corr_layout<T>(g.n[1], g.n[2], nsb);
         if (L.total > 200 * 1024) return false;
-        if (L.total > 48 * 1024)
-            cudaFuncSetAttribute(k_subbox_corr_planes<T, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total);
+        allow_smem(k_subbox_corr_planes<T, W>, L.total);
         k_subbox_corr_planes<T, W><<<dim3((unsigned)npair, (unsigned)W), SBC_THREADS, L.total, st>>>(g, nmodels, nfield, pairs, x, wc);
         return true;
     }
@@ -528,10 +527,10 @@ ds_status subbox_run(ds_model *M, const ds_qgrid *q, const ds_opts *o, T *d_out,
         const size_t sm = ((size_t)p.dres[2] * nsite + (size_t)nsite * 128) * sizeof(C);
         dim3 grid((unsigned)ktiles, (unsigned)(d12 * s3));
         if (NC == 1) {
-            if (sm > 48 * 1024) cudaFuncSetAttribute(k_subbox_res<T, 1, D3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+            allow_smem(k_subbox_res<T, 1, D3>, sm);
             k_subbox_res<T, 1, D3><<<grid, 128, sm, st>>>(p, S, s3);
         } else {
-            if (sm > 48 * 1024) cudaFuncSetAttribute(k_subbox_res<T, 3, D3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+            allow_smem(k_subbox_res<T, 3, D3>, sm);
             k_subbox_res<T, 3, D3><<<grid, 128, sm, st>>>(p, S, s3);
         }
         count_launches(1);

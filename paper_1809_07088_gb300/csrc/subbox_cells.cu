@@ -416,7 +416,7 @@ template <typename T, int KIND, bool LINE, bool WGT> void launch_rows(const SxPa
         // atoms of a row (<= 32 KB: n3 <= 128, nsite <= 16) and, for line sums, its first amplitudes
         const size_t sm = sizeof(float4) * p.n3 * maxs +
                           (LINE ? sizeof(c_t<T>) * (p.nsb - 1) * (KIND == SB_SPIN ? 3 : 1) * SX_T : 0);
-        if (sm > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        allow_smem(kern, sm);
         kern<<<grid, SX_T, sm, st>>>(p);
         count_launches(1);
     };

@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_taylor_sf(const __grid_constan
 
 template <typename T, int ZR, int NT> static void launch_sf_nt(const RecombParams<T> &p, cudaStream_t s) {
     const SFLayout L = sf_layout(ZR, p.nsite, p.sf.xpad, p.sf.ymax, p.sf.ngroups, sizeof(c_t<T>));
-    cudaFuncSetAttribute(k_taylor_sf<T, ZR, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total);
+    allow_smem(k_taylor_sf<T, ZR, NT>, L.total);
     dim3 grid((unsigned)p.g.ncell_h, 2);
     k_taylor_sf<T, ZR, NT><<<grid, NT, L.total, s>>>(p);
     count_launches(1);

@@ -125,3 +125,34 @@ def test_subbox_points_mean_term_of_an_undisplaced_crystal(ctx, prec, tag):
     org = syn.random_origins(rng, 1, m.cells, 360)
     got, _ = to_library(ctx, m).subbox_points(hkl, org, disorder=2, mode=1, precision=prec, subbox_n=2)
     assert np.all(got == 0.0)
+
+
+def test_shared_memory_limit_of_a_kernel_is_not_lowered_by_another_request(ctx):
+    """Two threads ask for sub-box volumes of the same box width whose planes take different amounts of
+    shared memory, both above the default limit: neither request's launch fails for the other's."""
+    import threading
+    import torch
+    lms, grids = [], []
+    for n in (100, 120):
+        m = syn.small_case(syn.OCC, cells=(4, n, n), nsite=1, nmodels=1, seed=243,
+                           qgrid=syn.QGrid(h0=(0.0, 0.0, 0.0), step=(0.25, 1.0 / n, 1.0 / n), count=(2, 2, 2)))
+        lms.append(to_library(ctx, m))
+        grids.append(qgrid_tuple(m.qgrid))
+    errors = []
+
+    def loop(i):
+        out = torch.empty((2, 2, 2), device="cuda")
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for _ in range(1500):
+                    lms[i].intensity(grids[i], out=out, disorder=0, mode=1, precision=1, smoothing=2, subbox_n=2)
+        except Exception as e:  # noqa: BLE001
+            errors.append(repr(e))
+
+    ts = [threading.Thread(target=loop, args=(i,)) for i in range(2)]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    torch.cuda.synchronize()
+    assert not errors
