@@ -247,6 +247,20 @@ void serving_shutdown(ds_ctx *ctx) {
     ctx->worker_started = false;
 }
 
+// A job leaves the table under the lock and its events are read and destroyed after the lock is released: a
+// completion callback waits for ctx->mu, and a driver call of another thread (an allocation, a launch that
+// has to resize local memory) may wait for that callback with the driver's own lock held, so a thread that
+// called the driver while holding ctx->mu could close the circle.
+static void forget(ds_ctx *ctx, ServeJob *j, std::unique_lock<std::mutex> &lk) {
+    ctx->jobs.erase(j->ticket);
+    lk.unlock();
+}
+static void free_job(ServeJob *j) {
+    cudaEventDestroy(j->e0);
+    cudaEventDestroy(j->e1);
+    delete j;
+}
+
 extern "C" ds_status ds_submit(ds_model *M, const ds_qgrid *q, const ds_opts *o, void *out, uint64_t *ticket) {
     if (!M) return DS_ERR_ARG;
     ds_ctx *ctx = M->ctx;
@@ -300,10 +314,8 @@ extern "C" ds_status ds_submit(ds_model *M, const ds_qgrid *q, const ds_opts *o,
         lk.lock();
         if (rc != DS_OK) {
             ctx->plan_free.push_back(j->plan_slot);
-            ctx->jobs.erase(j->ticket);
-            cudaEventDestroy(j->e0);
-            cudaEventDestroy(j->e1);
-            delete j;
+            forget(ctx, j, lk);
+            free_job(j);
             return rc == DS_ERR_CUDA ? ds_fail(ctx, rc, "planning launch failed") : rc;
         }
     } else {
@@ -316,10 +328,8 @@ extern "C" ds_status ds_submit(ds_model *M, const ds_qgrid *q, const ds_opts *o,
         ws.release();
         lk.lock();
         if (rc != DS_OK) {
-            ctx->jobs.erase(j->ticket);
-            cudaEventDestroy(j->e0);
-            cudaEventDestroy(j->e1);
-            delete j;
+            forget(ctx, j, lk);
+            free_job(j);
             return rc;
         }
         j->has_hint = true;
@@ -336,14 +346,9 @@ extern "C" ds_status ds_submit(ds_model *M, const ds_qgrid *q, const ds_opts *o,
     return DS_OK;
 }
 
-// fills info of a finished job, returns its status and forgets it.  The job leaves the table under the
-// lock and its events are read and destroyed after the lock is released: a completion callback waits
-// for ctx->mu, and a driver call of another thread (an allocation, a launch that has to resize local
-// memory) may wait for that callback with the driver's own lock held, so a thread that called the
-// driver while holding ctx->mu could close the circle.
+// fills info of a finished job, returns its status and forgets it
 static ds_status finish(ds_ctx *ctx, ServeJob *j, ds_result_info *info, std::unique_lock<std::mutex> &lk) {
-    ctx->jobs.erase(j->ticket);
-    lk.unlock();
+    forget(ctx, j, lk);
     ds_status st = j->status;
     if (info) {
         *info = j->info;
@@ -352,9 +357,7 @@ static ds_status finish(ds_ctx *ctx, ServeJob *j, ds_result_info *info, std::uni
         info->latency_ms = 1e3 * (j->t_done - j->t_submit);
         if (j->o.disorder == DS_DISP && j->xmax >= 0) info->x_max = j->xmax;
     }
-    cudaEventDestroy(j->e0);
-    cudaEventDestroy(j->e1);
-    delete j;
+    free_job(j);
     return st;
 }
 

@@ -1,6 +1,9 @@
 """Rules of the host code that need no GPU."""
+import os
 import re
 import subprocess
+
+import pytest
 
 
 def _symbols():
@@ -15,3 +18,24 @@ def test_atom_count_of_the_corner_maxima_is_64_bit():
     names = set(re.findall(r"_ZN2ds11corner_xmaxE\w+", _symbols()))
     assert names
     assert all(re.match(r"_ZN2ds11corner_xmaxEx", n) for n in names)
+
+
+@pytest.fixture(scope="module")
+def serving_host(tmp_path_factory):
+    """serving.cu linked with stand-ins for the CUDA runtime (serving_host.cu)."""
+    from paper_1809_07088_gb300 import build
+    build.build()
+    exe = str(tmp_path_factory.mktemp("serving") / "serving_host")
+    here = os.path.dirname(os.path.abspath(__file__))
+    cmd = [build._nvcc(), *build.ARCH, *build.FLAGS, "-cudart", "none", os.path.join(here, "serving_host.cu"),
+           os.path.join(build.OUT, "serving.o"), "-o", exe, "-lpthread"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    return exe
+
+
+@pytest.mark.parametrize("case", ["planning_fails", "planning_fails_without_a_slot"])
+def test_refused_request_frees_its_events_outside_the_lock(serving_host, case):
+    """A displacive request whose planning fails is dropped without a driver call under the context's lock."""
+    r = subprocess.run([serving_host, case], capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0, r.stderr
