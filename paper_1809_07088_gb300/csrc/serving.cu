@@ -375,11 +375,16 @@ extern "C" ds_status ds_wait(ds_ctx *ctx, uint64_t ticket, double timeout_s, ds_
     std::unique_lock<std::mutex> lk(ctx->mu);
     auto it = ctx->jobs.find(ticket);
     if (it == ctx->jobs.end()) return ds_fail(ctx, DS_ERR_ARG, "unknown ticket %llu", (unsigned long long)ticket);
-    ServeJob *j = it->second;
+    // another thread may take the result while this one waits: the job is looked up again each time
     const auto deadline = std::chrono::steady_clock::now() + std::chrono::duration<double>(timeout_s > 0 ? timeout_s : 0);
-    if (!ctx->cv.wait_until(lk, deadline, [&] { return j->done; }))
+    auto settled = [&] {
+        it = ctx->jobs.find(ticket);
+        return it == ctx->jobs.end() || it->second->done;
+    };
+    if (!ctx->cv.wait_until(lk, deadline, settled))
         return ds_fail(ctx, DS_ERR_TIMEOUT, "ticket %llu not finished after %.3f s", (unsigned long long)ticket, timeout_s);
-    return finish(ctx, j, info, lk);
+    if (it == ctx->jobs.end()) return ds_fail(ctx, DS_ERR_ARG, "unknown ticket %llu", (unsigned long long)ticket);
+    return finish(ctx, it->second, info, lk);
 }
 
 extern "C" ds_status ds_serving_pause(ds_ctx *ctx, int pause) {

@@ -107,6 +107,18 @@ int main(int argc, char **argv) {
         EXPECT(ds_submit(&model, &q, &o, &out, &t2) == DS_ERR_UNSUPPORTED);
         EXPECT(g_destroyed == 4);
         EXPECT(ctx.jobs.empty() && ctx.queue.empty());
+    } else if (!strcmp(which, "two_waiters")) {
+        o.taylor_order = 2;
+        ds_serving_pause(&ctx, 1);
+        EXPECT(ds_submit(&model, &q, &o, &out, &t) == DS_OK);
+        ds_status st[2];
+        std::thread w[2];
+        for (int i = 0; i < 2; ++i) w[i] = std::thread([&, i] { st[i] = ds_wait(&ctx, t, 10.0, nullptr); });
+        std::this_thread::sleep_for(std::chrono::milliseconds(300));   // both wait
+        ds_serving_pause(&ctx, 0);
+        for (int i = 0; i < 2; ++i) w[i].join();
+        EXPECT((st[0] == DS_OK && st[1] == DS_ERR_ARG) || (st[0] == DS_ERR_ARG && st[1] == DS_OK));
+        EXPECT(g_destroyed == 2);
     } else {
         return 2;
     }

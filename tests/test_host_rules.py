@@ -39,3 +39,10 @@ def test_refused_request_frees_its_events_outside_the_lock(serving_host, case):
     """A displacive request whose planning fails is dropped without a driver call under the context's lock."""
     r = subprocess.run([serving_host, case], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stderr
+
+
+def test_two_waiters_of_one_ticket(serving_host):
+    """The result of a ticket goes to one of two threads that wait for it; the other is told that the ticket is
+    unknown."""
+    r = subprocess.run([serving_host, "two_waiters"], capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0, r.stderr
