@@ -783,7 +783,8 @@ template <typename T, int NS, int ZPT, int MINB>
 __global__ void __launch_bounds__(DISP_KT * 32, MINB) k_recomb_disp(const __grid_constant__ RecombParams<T> p) {
     using C = c_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int kidx_s[DISP_KT], kconj_s[DISP_KT], site_s[NS];
+    __shared__ long long koff_s[DISP_KT];   // of monomial 0 within a site's spectra (the layout's division once per k)
+    __shared__ int kconj_s[DISP_KT], site_s[NS];
     const Geometry &g = p.g;
     const GridMap &gm = p.gm;
     const int nsite = p.nsite, nT = p.nT;
@@ -800,7 +801,7 @@ __global__ void __launch_bounds__(DISP_KT * 32, MINB) k_recomb_disp(const __grid
             const int f3 = kf % g.n[2], f2 = (kf / g.n[2]) % g.n[1], f1 = kf / (g.n[2] * g.n[1]);
             ki = half_index(g, f1, f2, f3, cj);
         }
-        kidx_s[threadIdx.x] = ki;
+        koff_s[threadIdx.x] = ki < 0 ? -1 : (long long)disp_spec_k(ki, nT, p.spec_kb);
         kconj_s[threadIdx.x] = cj;
     }
     if (threadIdx.x < NS) site_s[threadIdx.x] = threadIdx.x < nsite ? p.site_of[threadIdx.x] : -1;
@@ -885,6 +886,8 @@ __global__ void __launch_bounds__(DISP_KT * 32, MINB) k_recomb_disp(const __grid
         tops = p.sub_ops + p.sub_off[Pc];
     }
 
+    const size_t spec_site = disp_spec_site(g.ncell_h, nT, p.spec_kb);
+    const C *spec_m = p.spec + (size_t)p.model * nsite * spec_site;
     auto load_chunk = [&](int stage, int t0) {
         const int tc = min(DISP_TC, nTc - t0);
         C *dst = tile + stage * stage_elems;
@@ -893,10 +896,10 @@ __global__ void __launch_bounds__(DISP_KT * 32, MINB) k_recomb_disp(const __grid
             const int rest = idx / DISP_KT;
             const int tt = rest % DISP_TC, s = rest / DISP_TC;
             C *d = dst + ((size_t)kk * NS + s) * DISP_TC + tt;
-            const int ki = kidx_s[kk];
-            if (tt < tc && ki >= 0 && s < nsite) {
+            const long long ko = koff_s[kk];
+            if (tt < tc && ko >= 0 && s < nsite) {
                 const int t = tmap ? tmap[t0 + tt] : t0 + tt;
-                cp_async<sizeof(C)>(d, p.spec + ((size_t)p.model * nsite + site_s[s]) * disp_spec_site(g.ncell_h, nT, p.spec_kb) + disp_spec_k(ki, nT, p.spec_kb) + (size_t)t * p.spec_kb);
+                cp_async<sizeof(C)>(d, spec_m + site_s[s] * spec_site + ko + (size_t)t * p.spec_kb);
             } else {
                 *d = mk<T>(T(0), T(0));
             }
