@@ -16,9 +16,9 @@
 // cells), the Debye-Waller means from the same exponentials (DIFFUSE displacements), the boxes (grid:
 // points x origin chunks).  Partial sums are added in a fixed order.
 //
-// fcc 32^3 (131,072 atoms), 2516 origins, n_sb = 5, 40,401 points, FP32: 9.8 ms (29.5 ms box by box, at
-// 0.75 of the SFU rate); per chunk of 256 points the line sums take about 34 us (instruction issue 71 %),
-// the means 4, the boxes 22.
+// fcc 32^3 (131,072 atoms), 2516 origins, n_sb = 5, 40,401 points, FP32: 10.0 ms (29.5 ms box by box, at
+// 0.75 of the SFU rate); per chunk of 256 points the line sums take about 36 us, bound by instruction
+// issue, the means 4, the boxes 22.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -131,10 +131,11 @@ template <typename C> __device__ __forceinline__ C cmad(C x, C e, C a) {
 // Line sums (LINE) or plain amplitudes of whole rows of cells.  The row loop is unrolled by the ring
 // length, so the ring is indexed by constants.  Displacements: an atom costs three multiply-adds, one
 // reduction, one (sin, cos) pair, the product with its site's factor (four multiply-adds; formed in FP64
-// and rounded once, as box by box) and one add into its site's sum of cosines, the Debye-Waller mean.  Sites beyond nsite
-// (MAXS > nsite) are atoms of weight zero.  WGT: occupancies weight the displaced atoms.
-template <typename T, int KIND, int MAXS, bool LINE, bool WGT>
-__global__ void __launch_bounds__(SX_T, sizeof(T) == 4 && MAXS <= 4 && KIND != SB_SPIN ? 8 : 4) k_sx_rows(const __grid_constant__ SxParams<T> p) {
+// and rounded once, as box by box) and one add into its site's sum of cosines, the Debye-Waller mean.  WGT:
+// occupancies weight the displaced atoms.  GUARD: the sites beyond nsite are left out at run time (where a
+// site is dear: sines and cosines, FP64); without it they are atoms of weight zero.
+template <typename T, int KIND, int MAXS, bool LINE, bool WGT, bool GUARD>
+__global__ void __launch_bounds__(SX_T, KIND == SB_SPIN ? 4 : (sizeof(T) == 8 ? 2 : (MAXS <= 4 ? 8 : 4))) k_sx_rows(const __grid_constant__ SxParams<T> p) {
     using C = c_t<T>;
     constexpr int NC = KIND == SB_SPIN ? 3 : 1;
     extern __shared__ __align__(16) unsigned char sx_raw[];
@@ -194,6 +195,7 @@ __global__ void __launch_bounds__(SX_T, sizeof(T) == 4 && MAXS <= 4 && KIND != S
                         a[0] = mk<T>(T(0), T(0));
 #pragma unroll
                         for (int s = 0; s < MAXS; ++s) {
+                            if (GUARD && s >= nsite) break;
                             const float4 v = at[s];
                             const T t = fma(Qx, (T)v.x, fma(Qy, (T)v.y, Qz * (T)v.z));
                             T cs, sn;
@@ -210,6 +212,7 @@ __global__ void __launch_bounds__(SX_T, sizeof(T) == 4 && MAXS <= 4 && KIND != S
                         for (int c = 0; c < NC; ++c) a[c] = mk<T>(-K[c].x, -K[c].y);
 #pragma unroll
                         for (int s = 0; s < MAXS; ++s) {
+                            if (GUARD && s >= nsite) break;
                             const float4 v = at[s];
                             const T x[3] = {(T)v.x, (T)v.y, (T)v.z};
 #pragma unroll
@@ -420,23 +423,36 @@ template <typename T, int KIND, bool LINE, bool WGT> void launch_rows(const SxPa
         kern<<<grid, SX_T, sm, st>>>(p);
         count_launches(1);
     };
-    if constexpr (sizeof(T) == 4 && KIND == SB_DISP && LINE) {
-        // the SFU-bound case: no atom of weight zero up to six sites
-        switch (p.nsite) {
-        case 1: return go(k_sx_rows<T, KIND, 1, LINE, WGT>, 1);
-        case 2: return go(k_sx_rows<T, KIND, 2, LINE, WGT>, 2);
-        case 3: return go(k_sx_rows<T, KIND, 3, LINE, WGT>, 3);
-        case 5: return go(k_sx_rows<T, KIND, 5, LINE, WGT>, 5);
-        case 6: return go(k_sx_rows<T, KIND, 6, LINE, WGT>, 6);
-        default: break;
+    const int ns = p.nsite;
+    if constexpr (sizeof(T) == 4 && KIND == SB_DISP) {
+        // the SFU-bound case: instances of exactly nsite sites up to eight
+        if constexpr (LINE) {
+            switch (ns) {
+            case 1: return go(k_sx_rows<T, KIND, 1, LINE, WGT, false>, 1);
+            case 2: return go(k_sx_rows<T, KIND, 2, LINE, WGT, false>, 2);
+            case 3: return go(k_sx_rows<T, KIND, 3, LINE, WGT, false>, 3);
+            case 4: return go(k_sx_rows<T, KIND, 4, LINE, WGT, false>, 4);
+            case 5: return go(k_sx_rows<T, KIND, 5, LINE, WGT, false>, 5);
+            case 6: return go(k_sx_rows<T, KIND, 6, LINE, WGT, false>, 6);
+            case 7: return go(k_sx_rows<T, KIND, 7, LINE, WGT, false>, 7);
+            case 8: return go(k_sx_rows<T, KIND, 8, LINE, WGT, false>, 8);
+            default: break;
+            }
         }
+        ns == 16 ? go(k_sx_rows<T, KIND, 16, LINE, WGT, false>, 16) : go(k_sx_rows<T, KIND, 16, LINE, WGT, true>, 16);
+    } else {
+        // FP64 sums of occupancies and displacements leave idle sites out; moments (bound by the latency of
+        // their three rings) and FP32 occupancies run faster with idle sites of weight zero
+        constexpr bool G = sizeof(T) == 8 && KIND != SB_SPIN;
+        if constexpr (LINE || !G)
+            if (ns <= 4) return go(k_sx_rows<T, KIND, 4, LINE, WGT, G>, 4);
+        if constexpr (LINE) {
+            if (ns <= 8) return go(k_sx_rows<T, KIND, 8, LINE, WGT, G>, 8);
+        } else if (G && ns == 16) {
+            return go(k_sx_rows<T, KIND, 16, LINE, WGT, false>, 16);
+        }
+        go(k_sx_rows<T, KIND, 16, LINE, WGT, G>, 16);
     }
-    if constexpr (LINE) {
-        if (p.nsite <= 4) return go(k_sx_rows<T, KIND, 4, LINE, WGT>, 4);
-        if constexpr (sizeof(T) == 4)
-            if (p.nsite <= 8) return go(k_sx_rows<T, KIND, 8, LINE, WGT>, 8);
-    }
-    go(k_sx_rows<T, KIND, 16, LINE, WGT>, 16);
 }
 template <typename T, int KIND> void launch_rows(const SxParams<T> &p, bool line, const dim3 &grid, cudaStream_t st) {
     if constexpr (KIND == SB_DISP) {
@@ -475,31 +491,56 @@ template <typename T, int KIND> void run_kind(SxParams<T> p, double norm, int ch
     count_launches(1);
 }
 
+// Rule: the cheaper route by a cost model, picoseconds per point, of both routes measured on GB300 in both
+// precisions (768 pairs of times: 20^3 to 64^3 cells, 1 to 16 sites, boxes of 2^3 to 10^3 cells, 0.5 to 8
+// boxes per cell; 22,500 points in FP32, 2,500 in FP64).  Box by box: a term per cell of a box, and the
+// Debye-Waller pass of DIFFUSE displacements.  Shared: a term per cell, which grows with the box's width
+// (the ring of the line sums; amplitudes written and read again where the ring is too short) and with
+// the sites that are evaluated (FP64 moments: whole instances), and one per line sum read.
+// Few points leave the box-by-box launch short of blocks (fill < 1; measured for FP32 occupancies and moments:
+// 16^3 cells, six spins, 33 boxes of 8^3, 3600 points, fill 0.14: 1.00 box by box, 0.35 ms shared).
+// The line lies where the two are equal, 20^3 cells, n_sb = 5, four sites, box by box and shared: FP32
+// displacements 1.20 and 1.31 ms at 1.6 boxes per cell, 2.24 and 1.41 at 4; occupancies 0.54 and 0.77 ms,
+// 1.18 and 0.85; FP64 displacements 14.0 and 7.6 ms at 0.6; occupancies 0.91 and 1.30 ms at 0.6, 1.71 and
+// 1.34 at 1.6.  Where the rule shares, sharing was at most 6 % slower than box by box at any overlap between
+// the measured ones.  From 48^3 cells on the line sums of one block of points exceed the L2; sharing gains
+// there too (FP32, 64^3, four displaced sites, 2.5 boxes per cell, 1600 points: 7.5 and 2.4 ms).
+bool cells_cheaper(bool fp64, int kind, bool diffuse, int nsite, int nsb, double cells, double norigin, double fill) {
+    const int NC = kind == SB_SPIN ? 3 : 1;
+    const double ns = nsite, w = nsb;
+    const bool wide = nsb > SX_RING;
+    double box_cell, cell, line, dw = 0.0;
+    if (!fp64) {
+        line = kind == SB_SPIN ? 3.3 : 0.9;
+        if (kind == SB_DISP) box_cell = 0.4 + 0.5 * ns, cell = 3.8 + 0.5 * ns + 0.15 * std::max(0.0, ns - 6) + 0.1 * std::max(0.0, w - 5), dw = 0.48 * ns;
+        else if (kind == SB_OCC) box_cell = 0.9 + 0.145 * ns, cell = 2.2 + 0.28 * ns + 0.7 * std::max(0.0, w - 5);
+        else box_cell = 1.6 + 0.36 * ns, cell = 8.8 + 0.35 * ns + 0.55 * w;
+        if (wide) {
+            line = 0.9 * NC;
+            cell = (kind == SB_DISP ? 3.8 + 0.5 * ns : (kind == SB_OCC ? 2.2 + 0.28 * ns : 4.5 + 0.97 * ns)) + 2.3 * NC * w;
+        }
+    } else {
+        const double pad = nsite <= 4 ? 4 : (nsite <= 8 ? 8 : 16);
+        if (kind == SB_DISP) box_cell = 50 + 60 * ns, cell = 6 + 85 * ns + (wide ? 9.5 : 7.2) * w, line = 13, dw = 150 * ns;
+        else if (kind == SB_OCC) box_cell = 40 + 7 * ns, cell = 3 + 6.7 * ns + (wide ? 9.4 : 7.1) * w, line = 12;
+        else box_cell = 30 + 22 * ns, cell = wide ? 30 + 13 * pad + 33 * w : 80 + 15 * pad + 27 * w, line = 40;
+        if (wide) line = NC;
+    }
+    double by_box = norigin * w * w * w * box_cell + (diffuse ? dw * cells : 0.0);
+    if (!fp64 && kind != SB_DISP) by_box *= std::pow(fill, -0.4);
+    return cells * cell + norigin * w * w * line <= 0.95 * by_box;
+}
+
 }  // namespace
 
 template <typename T>
 bool subbox_cells_run(ds_model *M, int kind, const SbSite *d_sites, const int4 *d_org, long long norigin,
-                      const double *d_hkl, long long npts, const ds_opts *o, T *dout, Scratch &ws, cudaStream_t st) {
+                      const double *d_hkl, long long npts, const ds_opts *o, T *dout, double fill, Scratch &ws, cudaStream_t st) {
     using C = c_t<T>;
     ds_ctx *ctx = M->ctx;
     const int nsb = o->subbox_n, nsite = M->nsite, NC = kind == SB_SPIN ? 3 : 1;
     const double cells = (double)M->nmodels * M->n[0] * M->n[1] * M->n[2];
-    // Rule: the cheaper route by a cost model, picoseconds per point, fitted to both routes measured in
-    // FP32 on GB300 (22,500 points; 1, 4 and 16 sites; 65 to 1040 boxes of 3^3 to 10^3 cells).  Box by
-    // box: per cell of a box 0.4 + 0.5 nsite (displacements), 0.9 + 0.145 nsite (occupancies), 0.66 +
-    // 0.5 nsite (moments), and the Debye-Waller pass of DIFFUSE displacements.  Shared: per cell 3.8 +
-    // 0.5, 2.2 + 0.28, 4.5 + 0.97 nsite, 0.9 per line sum read (0.9 per component), 2.3 per amplitude
-    // read where the line sums take their own pass.  fcc 32^3, n_sb = 5, 150 x 150 points: 520 origins
-    // 4.9 (box by box) and 4.4 ms, 260 origins 3.2 and 4.3 ms; occupancies 1040 origins 4.4 and 2.9 ms,
-    // 520 origins 2.3 and 2.7 ms.
-    double box_cell, cell;
-    if (kind == SB_DISP) box_cell = 0.4 + 0.5 * nsite, cell = 3.8 + 0.5 * nsite;
-    else if (kind == SB_OCC) box_cell = 0.9 + 0.145 * nsite, cell = 2.2 + 0.28 * nsite;
-    else box_cell = 0.66 + 0.5 * nsite, cell = 4.5 + 0.97 * nsite;
-    double by_box = (double)norigin * nsb * nsb * nsb * box_cell;
-    if (kind == SB_DISP && o->mode == DS_DIFFUSE) by_box += 0.48 * nsite * cells;
-    const double by_cell = cells * (cell + (nsb > SX_RING ? 2.3 * NC * nsb : 0.0)) + (double)norigin * nsb * nsb * 0.9 * NC;
-    if (by_cell > 0.95 * by_box) return false;
+    if (!cells_cheaper(sizeof(T) == 8, kind, o->mode == DS_DIFFUSE, nsite, nsb, cells, (double)norigin, fill)) return false;
     // points per chunk: line sums (and amplitudes, for boxes wider than the ring) within SX_L2
     const size_t per_q = (size_t)cells * NC * sizeof(C) * (nsb > SX_RING ? 2 : 1);
     long long blocks = std::max<long long>(1, (long long)(SX_L2 / (per_q * SX_T)));
@@ -571,6 +612,6 @@ bool subbox_cells_run(ds_model *M, int kind, const SbSite *d_sites, const int4 *
 }
 
 template bool subbox_cells_run<float>(ds_model *, int, const SbSite *, const int4 *, long long, const double *, long long,
-                                      const ds_opts *, float *, Scratch &, cudaStream_t);
+                                      const ds_opts *, float *, double, Scratch &, cudaStream_t);
 template bool subbox_cells_run<double>(ds_model *, int, const SbSite *, const int4 *, long long, const double *,
-                                       long long, const ds_opts *, double *, Scratch &, cudaStream_t);
+                                       long long, const ds_opts *, double *, double, Scratch &, cudaStream_t);

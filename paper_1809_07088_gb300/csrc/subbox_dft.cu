@@ -780,8 +780,10 @@ ds_status run_subbox_points(ds_model *Mdl, const std::vector<int4> &org, const d
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, SB_THREADS, 0) != cudaSuccess ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess)
         return ds_fail(ctx, DS_ERR_CUDA, "occupancy query failed");
-    const long long per = origin_chunks(norigin, pblocks, (long long)std::max(1, per_sm) * std::max(1, nsm));
+    const long long resident = (long long)std::max(1, per_sm) * std::max(1, nsm);
+    const long long per = origin_chunks(norigin, pblocks, resident);
     const long long nchunk = (norigin + per - 1) / per;
+    const double fill = (double)norigin * pblocks / ((double)((pblocks * nchunk + resident - 1) / resident) * resident * per);
 
     if (Mdl->ready) cudaStreamWaitEvent(st, Mdl->ready, 0);  // uploads made on another stream
     Scratch ws(st);
@@ -800,7 +802,7 @@ ds_status run_subbox_points(ds_model *Mdl, const std::vector<int4> &org, const d
         (!hkl_dev && cudaMemcpyAsync((void *)d_hkl, hkl, sizeof(double) * 3 * npts, cudaMemcpyHostToDevice, st) != cudaSuccess))
         return ds_fail(ctx, DS_ERR_CUDA, "copy of the sub-box inputs failed");
     T *partial = nullptr, *dw = nullptr;
-    const bool shared = subbox_cells_run<T>(Mdl, kind, d_sites, d_org, norigin, d_hkl, npts, o, dout, ws, st);
+    const bool shared = subbox_cells_run<T>(Mdl, kind, d_sites, d_org, norigin, d_hkl, npts, o, dout, fill, ws, st);
     if (!shared) {
         partial = (T *)ws.get(sizeof(T) * nchunk * npts);
         if (kind == SB_DISP && o->mode == DS_DIFFUSE) dw = (T *)ws.get(sizeof(T) * nsite * npts);

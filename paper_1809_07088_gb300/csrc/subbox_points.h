@@ -45,7 +45,8 @@ __device__ __forceinline__ void cexp_acc(double2 &S, double2 phi, double2 iphi, 
 }
 
 // the shared-amplitude route (subbox_cells.cu): true when it took the request (its kernels are queued
-// on st); false leaves it to the box-by-box kernels
+// on st); false leaves it to the box-by-box kernels.  fill: the share of the resident blocks that their
+// launch would keep busy
 template <typename T>
 bool subbox_cells_run(ds_model *M, int kind, const SbSite *d_sites, const int4 *d_org, long long norigin,
-                      const double *d_hkl, long long npts, const ds_opts *o, T *dout, Scratch &ws, cudaStream_t st);
+                      const double *d_hkl, long long npts, const ds_opts *o, T *dout, double fill, Scratch &ws, cudaStream_t st);

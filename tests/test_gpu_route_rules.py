@@ -4,8 +4,8 @@ import numpy as np
 import pytest
 
 import synthetic as syn
-from oracle import core
-from _helpers import TOL, qgrid_tuple, to_library
+from oracle import core, noise
+from _helpers import TOL, qgrid_tuple, rel_err_of_peak, to_library
 
 pytestmark = pytest.mark.gpu
 PREC = [(0, "fp64"), (1, "fp32")]
@@ -125,6 +125,24 @@ def test_subbox_points_mean_term_of_an_undisplaced_crystal(ctx, prec, tag):
     org = syn.random_origins(rng, 1, m.cells, 360)
     got, _ = to_library(ctx, m).subbox_points(hkl, org, disorder=2, mode=1, precision=prec, subbox_n=2)
     assert np.all(got == 0.0)
+
+
+@pytest.mark.parametrize("prec,tag", PREC)
+@pytest.mark.parametrize("kind", ["occ", "spin", "disp"])
+@pytest.mark.parametrize("nsite,nsb", [(2, 2), (4, 9), (7, 8), (8, 3), (9, 2), (12, 9), (16, 4), (16, 9)])
+def test_subbox_points_shared_amplitudes_of_every_site_count(ctx, prec, tag, kind, nsite, nsb):
+    """Instances of exactly nsite sites, of more sites with the idle ones left out, and of boxes wider than the
+    register ring, with four boxes per cell (shared amplitudes) and one (box by box for most)."""
+    code = {"occ": syn.OCC, "spin": syn.SPIN, "disp": syn.DISP}[kind]
+    cells = (9, 10, 9) if nsb == 9 else (8, 9, 10)
+    m = syn.small_case(code, cells=cells, nsite=nsite, nmodels=1, seed=245)
+    lm = to_library(ctx, m)
+    rng = np.random.default_rng(34)
+    hkl = rng.uniform(-1.5, 1.5, (37, 3))
+    for ratio in (1, 4):
+        org = syn.random_origins(rng, 1, cells, max(2, ratio * int(np.prod(cells)) // nsb ** 3))
+        got, _ = lm.subbox_points(hkl, org, disorder=code, mode=1, precision=prec, subbox_n=nsb)
+        assert rel_err_of_peak(got, noise.subbox_intensity(m, kind, 1, nsb, hkl, org)) < TOL[tag]
 
 
 def test_shared_memory_limit_of_a_kernel_is_not_lowered_by_another_request(ctx):
