@@ -579,29 +579,34 @@ bool subbox_cells_run(ds_model *M, int kind, const SbSite *d_sites, const int4 *
     p.per_chunk = std::min<long long>(std::max<long long>(1, (norigin + want - 1) / want), 4096 / nsb);
     if ((norigin + p.per_chunk - 1) / p.per_chunk > 65535) return false;
     const int nochunk = (int)((norigin + p.per_chunk - 1) / p.per_chunk);
-    const size_t nk = (size_t)p.ldp, before = ws.total;
+    // one block, so that nothing is held when it cannot be had: the box-by-box route needs less
+    const size_t nk = (size_t)p.ldp;
     const bool mean_b = kind == SB_DISP && p.diffuse;
-    const size_t need = sizeof(C) * nk * (nsite + 3 + NC) + sizeof(T) * 3 * nk + (size_t)chunk_q * per_q +
-                        (mean_b ? sizeof(double2) * nk * nsite : 0) +
-                        (mean_b ? sizeof(T) * (size_t)(p.nrb + 1) * nsite * p.ld : 0) +
-                        sizeof(T) * (size_t)nochunk * npts;
-    if (before + need > ctx->budget) return false;
-    p.phi = (C *)ws.get(sizeof(C) * nk * nsite);
-    p.e = (C *)ws.get(sizeof(C) * nk * 3);
-    p.Q = (T *)ws.get(sizeof(T) * nk * 3);
-    if (mean_b) p.phiB = (double2 *)ws.get(sizeof(double2) * nk * nsite);
-    p.K = (C *)ws.get(sizeof(C) * nk * NC);
-    p.L = (C *)ws.get(sizeof(C) * (size_t)cells * NC * p.ld);
-    if (nsb > SX_RING) p.A = (C *)ws.get(sizeof(C) * (size_t)cells * NC * p.ld);
+    size_t need = 0;
+    std::vector<std::pair<void **, size_t>> parts;   // (pointer, offset)
+    auto part = [&](auto *&ptr, size_t count) {
+        parts.push_back({(void **)&ptr, need});
+        need += (count * sizeof(*ptr) + 255) & ~(size_t)255;
+    };
+    part(p.phi, nk * nsite);
+    part(p.e, nk * 3);
+    part(p.Q, nk * 3);
+    if (mean_b) part(p.phiB, nk * nsite);
+    part(p.K, nk * NC);
+    part(p.L, (size_t)cells * NC * p.ld);
+    if (nsb > SX_RING) part(p.A, (size_t)cells * NC * p.ld);
     if (mean_b) {
-        p.dwp = (T *)ws.get(sizeof(T) * (size_t)(p.nrb + 1) * nsite * p.ld);
-        p.dwm = p.dwp + (size_t)p.nrb * nsite * p.ld;
+        part(p.dwp, (size_t)p.nrb * nsite * p.ld);
+        part(p.dwm, (size_t)nsite * p.ld);
     }
-    p.partial = (T *)ws.get(sizeof(T) * (size_t)nochunk * npts);
-    if (ws.failed) {
-        ws.failed = false;   // the box-by-box route needs less
+    part(p.partial, (size_t)nochunk * npts);
+    if (ws.total + need > ctx->budget) return false;
+    char *block = (char *)ws.get(need);
+    if (!block) {
+        ws.failed = false;
         return false;
     }
+    for (auto &q : parts) *q.first = block + q.second;
     double norm = 1.0 / ((double)norigin * nsite * (double)nsb * nsb * nsb);
     if (kind == SB_SPIN) norm *= 0.07265;  // C of Eq. mag_intensity (barn)
     ProfScope ps(ctx, "subbox_cells", st);

@@ -20,18 +20,21 @@ def test_atom_count_of_the_corner_maxima_is_64_bit():
     assert all(re.match(r"_ZN2ds11corner_xmaxEx", n) for n in names)
 
 
-@pytest.fixture(scope="module")
-def serving_host(tmp_path_factory):
-    """serving.cu linked with stand-ins for the CUDA runtime (serving_host.cu)."""
+def _host_program(folder, source, obj):
+    """An object file of the library linked with stand-ins for the CUDA runtime (source)."""
     from paper_1809_07088_gb300 import build
     build.build()
-    exe = str(tmp_path_factory.mktemp("serving") / "serving_host")
-    here = os.path.dirname(os.path.abspath(__file__))
-    cmd = [build._nvcc(), *build.ARCH, *build.FLAGS, "-cudart", "none", os.path.join(here, "serving_host.cu"),
-           os.path.join(build.OUT, "serving.o"), "-o", exe, "-lpthread"]
+    exe = str(folder / source[:-3])
+    cmd = [build._nvcc(), *build.ARCH, *build.FLAGS, "-cudart", "none",
+           os.path.join(os.path.dirname(os.path.abspath(__file__)), source), os.path.join(build.OUT, obj), "-o", exe, "-lpthread"]
     r = subprocess.run(cmd, capture_output=True, text=True)
     assert r.returncode == 0, r.stderr
     return exe
+
+
+@pytest.fixture(scope="module")
+def serving_host(tmp_path_factory):
+    return _host_program(tmp_path_factory.mktemp("serving"), "serving_host.cu", "serving.o")
 
 
 @pytest.mark.parametrize("case", ["planning_fails", "planning_fails_without_a_slot"])
@@ -45,4 +48,10 @@ def test_two_waiters_of_one_ticket(serving_host):
     """The result of a ticket goes to one of two threads that wait for it; the other is told that the ticket is
     unknown."""
     r = subprocess.run([serving_host, "two_waiters"], capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0, r.stderr
+
+
+def test_shared_amplitude_route_holds_nothing_when_its_scratch_cannot_be_had(tmp_path):
+    exe = _host_program(tmp_path, "subbox_host.cu", "subbox_cells.o")
+    r = subprocess.run([exe], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stderr
