@@ -815,7 +815,7 @@ size_t request_footprint(const ds_model *M, const ds_qgrid *q, const ds_opts *o,
     }
     const size_t fb = std::max<size_t>(1, std::min<size_t>(nf, (512ull << 20) / (ce * g.ncell_h)));
     bytes += (nf + fb) * g.ncell_h * ce;
-    if (o->disorder == DS_DISP && nf * g.ncell_h * ce > SPEC_BLOCKED)
+    if (o->disorder == DS_DISP && spec_blocked(nf / (nmod * nsite), g.ncell_h, ce))
         bytes += nf * (disp_spec_site(g.ncell_h, 1, SPEC_KB) - g.ncell_h) * ce;
     const int hl = lanczos_like(o) ? lanczos_halo(o->lanczos_m, o->lanczos_mprime) : 0;
     if (lanczos_like(o)) bytes += 3 * (cnt[0] + 2 * hl) * (cnt[1] + 2 * hl) * (cnt[2] + 2 * hl) * es;
@@ -1074,7 +1074,7 @@ ds_status plan_and_run(ds_model *M, const ds_qgrid *q, const ds_opts *o, T *d_ou
 
     // per-site transforms (Section III)
     if (o->disorder == DS_DISP)
-        src.kb = p.spec_kb = sizeof(C) * (size_t)nf * g.ncell_h > SPEC_BLOCKED ? SPEC_KB : g.ncell_h;
+        src.kb = p.spec_kb = spec_blocked(Tn, g.ncell_h, sizeof(C)) ? SPEC_KB : g.ncell_h;
     const size_t nspec = o->disorder == DS_DISP ? (size_t)nmod * nsite * disp_spec_site(g.ncell_h, Tn, src.kb) : (size_t)nf * g.ncell_h;
     C *spec = (C *)ws.get(sizeof(C) * nspec);
     const size_t work_cap = 512ull << 20;

@@ -52,17 +52,19 @@ struct FieldSource {
     const void *real_buf; // SRC_REAL: [field][cell] (T)
 };
 
-// Spectra: [field][k] (k < ncell_h).  Taylor monomials whose spectra take more than SPEC_BLOCKED bytes:
+// Spectra: [field][k] (k < ncell_h).  Taylor monomials whose spectra take more than SPEC_BLOCKED bytes a site:
 // [model][site][k / kb][monomial][k % kb], kb = SPEC_KB (kb = ncell_h is the plain layout).  The
-// recombination reads every monomial of one k: with the field index outermost these are reads one
-// field (1 MB at 64^3) apart, each on a page of its own, at about 10^10 a second on GB300 whatever
-// their width; with 32 k in the innermost run they lie within 1.4 MB (5456 monomials), and the
-// transforms still store whole 256-byte runs.  perovskite 64^3, order 30 (29.5 GB): recombination
-// 90.3 -> 76.3 ms, transforms 29.6 -> 29.2 ms; fcc 32^3 (3.0 GB): 4.75 -> 4.40 ms, 1.90 -> 1.98 ms.
-// Spectra near the size of the L2 gain nothing and the stores cost more (fcc 16^3, 130 MB: the volume
-// 493 us plain, 507 us blocked).
+// recombination reads every monomial of one k, site by site: with the field index outermost these are
+// reads one field (1 MB at 64^3) apart, each on a page of its own, at about 10^10 a second on GB300
+// whatever their width; with 32 k in the innermost run they lie within 1.4 MB (5456 monomials), and the
+// transforms still store whole 256-byte runs.  perovskite 64^3, order 30 (5.9 GB a site): recombination
+// 90.3 -> 76.3 ms, transforms 29.6 -> 29.2 ms; fcc 32^3 (760 MB): 4.75 -> 4.40 ms, 1.90 -> 1.98 ms.
+// What the reads of one site span decides, not the size of all spectra.  Whole volumes, plain and blocked,
+// by the span: 42 MB (16^3, 16 sites) 1.92 and 1.99 ms, 192 MB (20^3) 3.09 and 3.16, 260 MB (36^3) 4.23 and
+// 4.25, 309 MB (64^3, one site) 3.02 and 2.99, 453 MB (36^3) 7.02 and 6.92, 513 MB (28^3) 2.24 and 2.11.
 constexpr int SPEC_KB = 32;
-constexpr size_t SPEC_BLOCKED = 512u << 20;
+constexpr size_t SPEC_BLOCKED = 300u << 20;
+inline bool spec_blocked(size_t nT, size_t ncell_h, size_t elem) { return nT * ncell_h * elem > SPEC_BLOCKED; }
 __host__ __device__ __forceinline__ size_t disp_spec_site(int ncell_h, int nT, int kb) {   // elements per (model, site)
     return (size_t)((ncell_h + kb - 1) / kb) * kb * nT;
 }

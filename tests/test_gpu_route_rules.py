@@ -145,6 +145,23 @@ def test_subbox_points_shared_amplitudes_of_every_site_count(ctx, prec, tag, kin
         assert rel_err_of_peak(got, noise.subbox_intensity(m, kind, 1, nsb, hkl, org)) < TOL[tag]
 
 
+@pytest.mark.parametrize("prec,tag", PREC)
+@pytest.mark.parametrize("kernel", [1, 2])
+def test_blocked_taylor_spectra_with_a_last_block_of_less_than_32(ctx, prec, tag, kernel):
+    """Monomial spectra above the size (300 MB a site) from which they are stored by blocks of 32 k, on unequal
+    axes whose half spectrum (23,100 values) ends in a block of 28, for two supercells of three sites: both
+    Taylor kernels, with and without the mean, against the direct sum.  The order is far above what |Q.u| needs."""
+    m = syn.small_case(syn.DISP, cells=(35, 30, 42), nsite=3, nmodels=2, seed=246, sigma=0.04)
+    m.qgrid = syn.QGrid(h0=(-1.0 / 35, 29.0 / 30, -2.0 / 42), step=(1.0 / 35, 1.0 / 30, 1.0 / 42), count=(3, 3, 4))
+    lm = to_library(ctx, m)
+    for mode in (0, 1):
+        got, info = lm.intensity(qgrid_tuple(m.qgrid), disorder=2, mode=mode, precision=prec,
+                                 taylor_order=17 if prec == 0 else 22, taylor_kernel=kernel)
+        assert info["n_monomials"] * 23100 * (16 if prec == 0 else 8) > 300 << 20
+        want = core.displacive_intensity_direct(m, m.qgrid.hkl(), mode)
+        assert rel_err_of_peak(got, want) < TOL[tag]
+
+
 def test_shared_memory_limit_of_a_kernel_is_not_lowered_by_another_request(ctx):
     """Two threads ask for sub-box volumes of the same box width whose planes take different amounts of
     shared memory, both above the default limit: neither request's launch fails for the other's."""
