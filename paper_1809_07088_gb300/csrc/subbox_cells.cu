@@ -6,7 +6,8 @@
 //     A_R(Q) = sum_mu phi_mu(Q) a_{R,mu}(Q),   a = delta, M or delta exp(i Q.u),
 // carries no box, so it is formed once per cell and point instead of once per box; a box then costs
 //     F_o = sum_d1 e1^d1 sum_d2 e2^d2 L_{o + (d1, d2, 0)},   L_R = sum_d3 e3^d3 A_{R + (0, 0, d3)},
-// e_a = exp(2 pi i h_a), with cells wrapped and phases not (open boxes).  The line sums L are formed as
+// e_a = exp(2 pi i h_a), with cells wrapped and phases not (open boxes).  With tabulated powers the line
+// sums of the ring leave out the phase e3^(nsb - 1), common to every box of a point.  The line sums L are formed as
 // the cells of a row are walked (the last eight amplitudes stay in registers), so a box reads n_sb^2
 // values per point.  For displacements the bound moves from one SFU (sin, cos) pair per atom and box to
 // one per atom, plus the L2 traffic of the line sums.
@@ -16,9 +17,9 @@
 // cells), the Debye-Waller means from the same exponentials (DIFFUSE displacements), the boxes (grid:
 // points x origin chunks).  Partial sums are added in a fixed order.
 //
-// fcc 32^3 (131,072 atoms), 2516 origins, n_sb = 5, 40,401 points, FP32: 10.0 ms (29.5 ms box by box, at
-// 0.75 of the SFU rate); per chunk of 256 points the line sums take about 36 us, bound by instruction
-// issue, the means 4, the boxes 22.
+// fcc 32^3 (131,072 atoms), 2516 origins, n_sb = 5, 40,401 points, FP32: 10.5 ms (29.5 ms box by box, at
+// 0.75 of the SFU rate); per chunk of 256 points, cold caches, the line sums take 35.5 us (instruction issue
+// 72 %, 96 registers, five CTAs per SM), the mean 6.5, the boxes 26.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -37,6 +38,11 @@ constexpr size_t SX_MOST = 1024u << 20;       // and at most, for one block of p
 constexpr long long SX_PREP = 65536;          // points whose constants are held at once
 constexpr int SX_RING = 8;                    // amplitudes of a row kept in registers
 
+// FP32 displacements take tabulated powers of the cell phases, each formed in FP64 and rounded once: powers of a rounded
+// phase drift by a rounding per cell (2.5e-7 of the result against 1.0e-7, boxes of 5^3, TOTAL), which the box-by-box
+// kernel's per-atom phases do not.  Its occupancies and moments advance a rounded phase too, as here.
+template <typename T, int KIND> constexpr bool sx_tab() { return sizeof(T) == 4 && KIND == SB_DISP; }
+
 template <typename T> struct SxParams {
     int nsite, nsb, n1, n2, n3, ncell, nmodels, diffuse;
     const SbSite *site;
@@ -51,12 +57,14 @@ template <typename T> struct SxParams {
     long long ldp;                  // stride of the constants
     double recip[9];
     c_t<T> *phi;                    // [site][ldp]: phi_mu
-    c_t<T> *e;                      // [axis][ldp]
+    c_t<T> *e;                      // [axis][u][ldp]: e_axis^u for u < 8, e_axis^8
     T *Q;                           // [axis][ldp]: Q / 2 pi (cycles per A) for displacements, Q for moments
-    double2 *phiB;                  // displacements: [site][ldp]: phi_mu times the box sum of exp(2 pi i Q.d)
+    double2 *phiB;                  // displacements: [site][ldp]: phi_mu exp(2 pi i off) times the box sum of exp(2 pi i Q.d)
+    T off, off_c, off_s;            // displacements: phase added to every Q.u (cycles), its cosine and sine
     c_t<T> *K;                      // occupancies, moments: mean amplitude [comp][ldp]
     c_t<T> *A, *L;                  // [comp][model cell][ld]; A: amplitudes where the line sums take their own pass
-    T *dwp, *dwm;                   // [row block][site][ld]: sums of w cos(Q.u); [site][ld]: their mean
+    T *dwp;                         // [row block][site][ld]: sums of w cos(Q.u)
+    c_t<T> *KB;                     // [ld]: the mean amplitude of a box
     int rows_per, nrb;              // rows of cells per block, row blocks
     const int4 *origins;
     long long norigin, per_chunk;
@@ -76,22 +84,27 @@ template <typename T, int KIND> __global__ void __launch_bounds__(SX_T) k_sx_pre
         p.Q[a * p.ldp + j] = (T)(KIND == SB_DISP ? Qd[a] / TWO_PI_D : Qd[a]);
     }
     const double s2 = (Qd[0] * Qd[0] + Qd[1] * Qd[1] + Qd[2] * Qd[2]) / (FOUR_PI_D * FOUR_PI_D);
-    double Br = 1.0, Bi = 0.0;
+    double Br = 1.0, Bi = 0.0, lr = 1.0, li = 0.0;   // (lr, li): what the line sums leave out, e_3^-(nsb - 1)
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         double sn, cs;
         sincospi(2.0 * frac_w(h[a]), &sn, &cs);
-        p.e[a * p.ldp + j] = mk<T>((T)cs, (T)sn);
         double xr = 1.0, xi = 0.0, sr = 0.0, si = 0.0;   // sum_d e^d
-        for (int d = 0; d < p.nsb; ++d) {
-            sr += xr;
-            si += xi;
+        for (int d = 0; d < max(p.nsb, SX_RING + 1); ++d) {
+            if (d <= SX_RING) p.e[(a * (SX_RING + 1) + d) * p.ldp + j] = mk<T>((T)xr, (T)xi);
+            if (d < p.nsb) sr += xr, si += xi;
+            if (sx_tab<T, KIND>() && a == 2 && d == p.nsb - 1 && p.nsb <= SX_RING) lr = xr, li = -xi;
             const double t = xr * cs - xi * sn;
             xi = xr * sn + xi * cs;
             xr = t;
         }
         const double t = Br * sr - Bi * si;
         Bi = Br * si + Bi * sr;
+        Br = t;
+    }
+    {
+        const double t = Br * lr - Bi * li;
+        Bi = Br * li + Bi * lr;
         Br = t;
     }
     constexpr int NC = KIND == SB_SPIN ? 3 : 1;
@@ -105,6 +118,7 @@ template <typename T, int KIND> __global__ void __launch_bounds__(SX_T) k_sx_pre
         double sn, cs;
         sincospi(2.0 * t, &sn, &cs);
         p.phi[s * p.ldp + j] = mk<T>((T)(f * cs), (T)(f * sn));
+        if (KIND == SB_DISP) sincospi(2.0 * (t + (double)p.off), &sn, &cs);
         if (KIND == SB_DISP && p.diffuse) p.phiB[s * p.ldp + j] = make_double2(f * cs * Br - f * sn * Bi, f * cs * Bi + f * sn * Br);
         if (KIND != SB_DISP && p.diffuse) {
 #pragma unroll
@@ -131,11 +145,15 @@ template <typename C> __device__ __forceinline__ C cmad(C x, C e, C a) {
 // Line sums (LINE) or plain amplitudes of whole rows of cells.  The row loop is unrolled by the ring
 // length, so the ring is indexed by constants.  Displacements: an atom costs three multiply-adds, one
 // reduction, one (sin, cos) pair, the product with its site's factor (four multiply-adds; formed in FP64
-// and rounded once, as box by box) and one add into its site's sum of cosines, the Debye-Waller mean.  WGT:
+// and rounded once, as box by box) and two adds into its site's sum, the Debye-Waller mean.
+// DIFFUSE FP32 requests add the phase off = 1/16 cycle to every atom: the fast sine falls short by about
+// 1.2e-7 on either side of the multiples of a quarter, 6e-7 of sin(Q.u) where |Q.u| stays below 0.3, and what
+// is left of an intensity without its mean is sin(Q.u) (4.3e-7 of it without the phase, boxes of 2^3).  At 1/16
+// the error has no slope.  The phase is common to F and K B.  TOTAL needs none: cosines near 1 are exact.  WGT:
 // occupancies weight the displaced atoms.  GUARD: the sites beyond nsite are left out at run time (where a
 // site is dear: sines and cosines, FP64); without it they are atoms of weight zero.
 template <typename T, int KIND, int MAXS, bool LINE, bool WGT, bool GUARD>
-__global__ void __launch_bounds__(SX_T, KIND == SB_SPIN ? 4 : (sizeof(T) == 8 ? 2 : (MAXS <= 4 ? 8 : 4))) k_sx_rows(const __grid_constant__ SxParams<T> p) {
+__global__ void __launch_bounds__(SX_T, KIND == SB_SPIN ? 4 : (sizeof(T) == 8 ? (KIND == SB_DISP && MAXS > 8 ? 2 : 4) : (MAXS <= 4 ? (KIND == SB_DISP ? 5 : 8) : 4))) k_sx_rows(const __grid_constant__ SxParams<T> p) {
     using C = c_t<T>;
     constexpr int NC = KIND == SB_SPIN ? 3 : 1;
     extern __shared__ __align__(16) unsigned char sx_raw[];
@@ -145,13 +163,23 @@ __global__ void __launch_bounds__(SX_T, KIND == SB_SPIN ? 4 : (sizeof(T) == 8 ? 
     const int ql = blockIdx.x * SX_T + tid;
     const long long j = p.q0 + ql;                     // < ldp: chunks are whole blocks
     C phi[MAXS];
-    T wsum[KIND == SB_DISP ? MAXS : 1];
+    C wsum[KIND == SB_DISP ? MAXS : 1];
 #pragma unroll
     for (int s = 0; s < MAXS; ++s) {
         phi[s] = s < nsite ? p.phi[s * p.ldp + j] : mk<T>(T(0), T(0));
-        if (KIND == SB_DISP) wsum[KIND == SB_DISP ? s : 0] = T(0);
+        if (KIND == SB_DISP) wsum[KIND == SB_DISP ? s : 0] = mk<T>(T(0), T(0));
     }
-    const C e3 = p.e[2 * p.ldp + j];
+    constexpr bool TAB = sx_tab<T, KIND>();
+    const C e3 = p.e[(2 * (SX_RING + 1) + 1) * p.ldp + j];
+    C q3[TAB ? SX_RING : 1];   // e_3^-i of the ring
+    if (LINE && TAB) {
+#pragma unroll
+        for (int i = 0; i < SX_RING; ++i) {
+            C q = i < nsb ? p.e[(2 * (SX_RING + 1) + i) * p.ldp + j] : mk<T>(T(0), T(0));
+            q.y = -q.y;
+            q3[TAB ? i : 0] = q;
+        }
+    }
     T Qx = T(0), Qy = T(0), Qz = T(0);
     C K[NC];
     if (KIND == SB_DISP) {
@@ -197,14 +225,16 @@ __global__ void __launch_bounds__(SX_T, KIND == SB_SPIN ? 4 : (sizeof(T) == 8 ? 
                         for (int s = 0; s < MAXS; ++s) {
                             if (GUARD && s >= nsite) break;
                             const float4 v = at[s];
-                            const T t = fma(Qx, (T)v.x, fma(Qy, (T)v.y, Qz * (T)v.z));
+                            const T t = fma(Qx, (T)v.x, fma(Qy, (T)v.y, fma(Qz, (T)v.z, p.off)));
                             T cs, sn;
                             sincos_cycles(frac_w(t), cs, sn);
                             if (WGT) {
                                 cs *= (T)v.w;
                                 sn *= (T)v.w;
                             }
-                            wsum[KIND == SB_DISP ? s : 0] += cs;
+                            C &ws = wsum[KIND == SB_DISP ? s : 0];
+                            ws.x += cs;
+                            ws.y += sn;
                             a[0] = cmad(phi[s], mk<T>(cs, sn), a[0]);
                         }
                     } else {
@@ -242,7 +272,8 @@ __global__ void __launch_bounds__(SX_T, KIND == SB_SPIN ? 4 : (sizeof(T) == 8 ? 
 #pragma unroll
                             for (int i = 1; i < SX_RING; ++i) {
                                 if (i >= nsb) break;
-                                l = cmad(l, e3, h[c][(u - i + SX_RING) % SX_RING]);
+                                const C hv = h[c][(u - i + SX_RING) % SX_RING];
+                                l = TAB ? cmad(q3[TAB ? i : 0], hv, l) : cmad(l, e3, hv);
                             }
                         }
                         d0[c * cstride + (ptrdiff_t)u * p.ld] = l;
@@ -256,48 +287,91 @@ __global__ void __launch_bounds__(SX_T, KIND == SB_SPIN ? 4 : (sizeof(T) == 8 ? 
         }
     }
     if (KIND == SB_DISP && p.diffuse) {
+        // sum of w cos(Q.u) = Re[exp(-2 pi i off) sum of w exp(i Q.u + 2 pi i off)]
 #pragma unroll
         for (int s = 0; s < MAXS; ++s)
-            if (s < nsite) p.dwp[((size_t)blockIdx.y * nsite + s) * p.ld + ql] = wsum[KIND == SB_DISP ? s : 0];
+            if (s < nsite) {
+                const C ws = wsum[KIND == SB_DISP ? s : 0];
+                p.dwp[((size_t)blockIdx.y * nsite + s) * p.ld + ql] = fma(ws.x, p.off_c, ws.y * p.off_s);
+            }
     }
 }
 
 // line sums of boxes wider than the register ring, from the amplitudes
-template <typename T> __global__ void __launch_bounds__(SX_T) k_sx_line(const __grid_constant__ SxParams<T> p, int nc) {
+template <typename T, bool TAB> __global__ void __launch_bounds__(SX_T) k_sx_line(const __grid_constant__ SxParams<T> p, int nc) {
     using C = c_t<T>;
     const int ql = blockIdx.x * SX_T + threadIdx.x;
-    const C e3 = p.e[2 * p.ldp + p.q0 + ql];
+    const C e3 = p.e[(2 * (SX_RING + 1) + 1) * p.ldp + p.q0 + ql];
+    C pw[SX_RING + 1];   // e_3^u
+#pragma unroll
+    for (int u = 0; u <= SX_RING; ++u) pw[u] = !TAB ? e3 : p.e[(2 * (SX_RING + 1) + u) * p.ldp + p.q0 + ql];
     const size_t cells = (size_t)p.nmodels * p.ncell;
     for (size_t i = blockIdx.y; i < cells * nc; i += gridDim.y) {
         const size_t row = i / p.n3;
         const int r3 = (int)(i - row * p.n3);
         const C *a = p.A + row * p.n3 * p.ld + ql;
         C l = mk<T>(T(0), T(0));
-        for (int d = p.nsb - 1; d >= 0; --d) {
-            int w = r3 + d;
-            if (w >= p.n3) w -= p.n3;
-            l = cmad(l, e3, a[(size_t)w * p.ld]);
+        if (TAB) {
+            for (int d0 = (p.nsb - 1) / SX_RING * SX_RING; d0 >= 0; d0 -= SX_RING) {
+                l = cmul(l, pw[SX_RING]);
+#pragma unroll
+                for (int u = 0; u < SX_RING; ++u) {
+                    if (d0 + u >= p.nsb) break;
+                    int w = r3 + d0 + u;
+                    if (w >= p.n3) w -= p.n3;
+                    l = cmad(pw[u], a[(size_t)w * p.ld], l);
+                }
+            }
+        } else {
+            for (int d = p.nsb - 1; d >= 0; --d) {
+                int w = r3 + d;
+                if (w >= p.n3) w -= p.n3;
+                l = cmad(l, e3, a[(size_t)w * p.ld]);
+            }
         }
         p.L[i * p.ld + ql] = l;
     }
 }
 
-// <w cos(Q.u)>_mu of the chunk's points: the row blocks' sums, by 32 threads per point in a fixed order
-constexpr int SX_MB = 32;
-template <typename T> __global__ void __launch_bounds__(32 * SX_MB) k_sx_mean(const __grid_constant__ SxParams<T> p) {
-    __shared__ T red[SX_MB][33];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, s = blockIdx.y;
-    const int ql = blockIdx.x * 32 + lane;
+// K B of the chunk's points, K = sum_mu phi_mu <w cos(Q.u)>_mu: the row blocks' sums by slices of 8 points and 128
+// threads each, in a fixed order; K B in FP64, rounded once (it cancels against F at Bragg positions)
+constexpr int SX_MP = 8, SX_MG = 128;
+template <typename T> __global__ void __launch_bounds__(SX_MP * SX_MG) k_sx_mean(const __grid_constant__ SxParams<T> p) {
+    __shared__ T red[SX_MG / 4][SX_MP + 1];
+    __shared__ double2 term[MAX_SITES][SX_MP];
+    const int tx = threadIdx.x % SX_MP, g = threadIdx.x / SX_MP, nsite = p.nsite;
+    const int nsl = (SX_MG / nsite) & ~3, s = g / nsl, sl = g - s * nsl;   // slices of a site, the thread's site and slice
+    const int ql = blockIdx.x * SX_MP + tx;
+    double2 pb = make_double2(0.0, 0.0);
+    if (g < nsite) pb = p.phiB[g * p.ldp + p.q0 + ql];
     T t = T(0);
-#pragma unroll 16
-    for (int b = w; b < p.nrb; b += SX_MB) t += p.dwp[((size_t)b * p.nsite + s) * p.ld + ql];
-    red[w][lane] = t;
-    __syncthreads();
-    if (w == 0) {
-        T sum = T(0);
+    if (s < nsite) {
+        const T *q = p.dwp + ((size_t)sl * nsite + s) * p.ld + ql;
+        const size_t step = (size_t)nsl * nsite * p.ld;
+        constexpr int NL = 16;   // loads in flight
+        for (int b = sl; b < p.nrb; b += NL * nsl, q += NL * step) {
+            T v[NL];
 #pragma unroll
-        for (int i = 0; i < SX_MB; ++i) sum += red[i][lane];
-        p.dwm[(size_t)s * p.ld + ql] = sum / (T)((double)p.nmodels * p.ncell);
+            for (int u = 0; u < NL; ++u) v[u] = b + u * nsl < p.nrb ? q[u * step] : T(0);
+#pragma unroll
+            for (int u = 0; u < NL; ++u) t += v[u];
+        }
+    }
+    t += __shfl_xor_sync(0xffffffffu, t, SX_MP);   // the four slices of a warp are of one site
+    t += __shfl_xor_sync(0xffffffffu, t, 2 * SX_MP);
+    if (g % 4 == 0) red[g / 4][tx] = t;
+    __syncthreads();
+    if (g < nsite) {
+        T sum = T(0);
+        for (int i = 0; i < nsl / 4; ++i) sum += red[g * (nsl / 4) + i][tx];
+        const double w = (double)(sum / (T)((double)p.nmodels * p.ncell));
+        term[g][tx] = make_double2(pb.x * w, pb.y * w);
+    }
+    __syncthreads();
+    if (g == 0) {
+        double kr = 0.0, ki = 0.0;
+        for (int i = 0; i < nsite; ++i) kr += term[i][tx].x, ki += term[i][tx].y;
+        p.KB[ql] = mk<T>((T)kr, (T)ki);
     }
 }
 
@@ -309,7 +383,9 @@ __global__ void __launch_bounds__(SX_T) k_sx_boxes(const __grid_constant__ SxPar
     constexpr int NC = KIND == SB_SPIN ? 3 : 1;
     constexpr int NB = SX_RING;
     extern __shared__ __align__(16) unsigned char sx_raw[];
-    int *off1 = (int *)sx_raw;                      // [origin][nsb]: element offset of (model, o1 + d1, 0, o3)
+    constexpr bool TAB = sx_tab<T, KIND>();
+    C *pw1 = (C *)sx_raw + threadIdx.x;             // TAB: [u][SX_T], e_1^u
+    int *off1 = (int *)((C *)sx_raw + (TAB ? SX_RING * SX_T : 0));   // [origin][nsb]: element offset of (model, o1 + d1, 0, o3)
     int *off2 = off1 + p.per_chunk * p.nsb;         // [origin][nsb]: of row o2 + d2 within a plane
     const int nsb = p.nsb;
     const int ql = blockIdx.x * SX_T + threadIdx.x;
@@ -325,24 +401,25 @@ __global__ void __launch_bounds__(SX_T) k_sx_boxes(const __grid_constant__ SxPar
         off1[i] = ((og.x * p.n1 + w1) * p.n2 * p.n3 + og.w) * p.ld;
         off2[i] = w2 * p.n3 * p.ld;
     }
-    const C e1 = p.e[j], e2 = p.e[p.ldp + j];
-    C pw[NB];   // e2^u
-    pw[0] = mk<T>(T(1), T(0));
+    // e_2^u below the box's width, and the eighth powers of wider boxes
+    const C e1 = p.e[p.ldp + j], e2 = p.e[(SX_RING + 2) * p.ldp + j];
+    C pw[NB], e1n = mk<T>(T(1), T(0)), e2n = e1n;
+    pw[0] = e1n;
 #pragma unroll
-    for (int u = 1; u < NB; ++u) pw[u] = cmul(pw[u - 1], e2);
-    const C e2n = cmul(pw[NB - 1], e2);
-    C KB = mk<T>(T(0), T(0));
-    if (KIND == SB_DISP && p.diffuse) {
-        // K B, K = sum_mu phi_mu <w cos(Q.u)>_mu: cancels against F at Bragg positions, so FP64, rounded once
-        double kr = 0.0, ki = 0.0;
-        for (int s = 0; s < p.nsite; ++s) {
-            const double2 pb = p.phiB[s * p.ldp + j];
-            const double w = (double)p.dwm[(size_t)s * p.ld + ql];
-            kr = fma(pb.x, w, kr);
-            ki = fma(pb.y, w, ki);
-        }
-        KB = mk<T>((T)kr, (T)ki);
+    for (int u = 1; u < NB; ++u) {
+        if (!TAB) pw[u] = cmul(pw[u - 1], e2);
+        else pw[u] = u < nsb ? p.e[(SX_RING + 1 + u) * p.ldp + j] : pw[0];
     }
+    if (TAB) {
+#pragma unroll
+        for (int u = 0; u < NB; ++u)
+            if (u < nsb) pw1[u * SX_T] = p.e[u * p.ldp + j];
+        if (nsb > NB) e1n = p.e[SX_RING * p.ldp + j], e2n = p.e[(2 * SX_RING + 1) * p.ldp + j];
+    } else {
+        e2n = cmul(pw[NB - 1], e2);
+    }
+    C KB = mk<T>(T(0), T(0));
+    if (KIND == SB_DISP && p.diffuse) KB = p.KB[ql];
     T Qv[3] = {T(0), T(0), T(0)};
     if (KIND == SB_SPIN)
 #pragma unroll
@@ -356,6 +433,10 @@ __global__ void __launch_bounds__(SX_T) k_sx_boxes(const __grid_constant__ SxPar
 #pragma unroll
         for (int c = 0; c < NC; ++c) F[c] = mk<T>(T(0), T(0));
         for (int d1 = nsb - 1; d1 >= 0; --d1) {
+            if (TAB && d1 % SX_RING == SX_RING - 1 && d1 < nsb - 1) {
+#pragma unroll
+                for (int c = 0; c < NC; ++c) F[c] = cmul(F[c], e1n);
+            }
             const C *pl = L + off1[oi * nsb + d1];
             C G[NC];
 #pragma unroll
@@ -384,7 +465,7 @@ __global__ void __launch_bounds__(SX_T) k_sx_boxes(const __grid_constant__ SxPar
                 }
             }
 #pragma unroll
-            for (int c = 0; c < NC; ++c) F[c] = cmad(F[c], e1, G[c]);
+            for (int c = 0; c < NC; ++c) F[c] = TAB ? cmad(pw1[(d1 % SX_RING) * SX_T], G[c], F[c]) : cmad(F[c], e1, G[c]);
         }
         T tot = T(0);
         if (KIND == SB_DISP) F[0] = csub(F[0], KB);
@@ -462,6 +543,7 @@ template <typename T, int KIND> void launch_rows(const SxParams<T> &p, bool line
 }
 
 template <typename T, int KIND> void run_kind(SxParams<T> p, double norm, int chunk_q, int nochunk, T *dout, cudaStream_t st) {
+    using C = c_t<T>;
     constexpr int NC = KIND == SB_SPIN ? 3 : 1;
     const bool line = p.nsb <= SX_RING;
     for (p.p0 = 0; p.p0 < p.npts; p.p0 += SX_PREP) {
@@ -475,14 +557,15 @@ template <typename T, int KIND> void run_kind(SxParams<T> p, double norm, int ch
             launch_rows<T, KIND>(p, line, rows, st);
             if (!line) {
                 const size_t lines = (size_t)p.nmodels * p.ncell * NC;
-                k_sx_line<T><<<dim3(qb, (unsigned)std::min<size_t>(lines, 16384)), SX_T, 0, st>>>(p, NC);
+                k_sx_line<T, sx_tab<T, KIND>()><<<dim3(qb, (unsigned)std::min<size_t>(lines, 16384)), SX_T, 0, st>>>(p, NC);
                 count_launches(1);
             }
             if (KIND == SB_DISP && p.diffuse) {
-                k_sx_mean<T><<<dim3(qb * (SX_T / 32), (unsigned)p.nsite), 32 * SX_MB, 0, st>>>(p);
+                k_sx_mean<T><<<qb * (SX_T / SX_MP), SX_MP * SX_MG, 0, st>>>(p);
                 count_launches(1);
             }
-            k_sx_boxes<T, KIND><<<dim3(qb, (unsigned)nochunk), SX_T, sizeof(int) * 2 * p.per_chunk * p.nsb, st>>>(p);
+            k_sx_boxes<T, KIND><<<dim3(qb, (unsigned)nochunk), SX_T,
+                                    (sx_tab<T, KIND>() ? sizeof(C) * SX_RING * SX_T : 0) + sizeof(int) * 2 * p.per_chunk * p.nsb, st>>>(p);
             count_launches(1);
         }
     }
@@ -500,11 +583,12 @@ template <typename T, int KIND> void run_kind(SxParams<T> p, double norm, int ch
 // Few points leave the box-by-box launch short of blocks (fill < 1; measured for FP32 occupancies and moments:
 // 16^3 cells, six spins, 33 boxes of 8^3, 3600 points, fill 0.14: 1.00 box by box, 0.35 ms shared).
 // The line lies where the two are equal, 20^3 cells, n_sb = 5, four sites, box by box and shared: FP32
-// displacements 1.20 and 1.31 ms at 1.6 boxes per cell, 2.24 and 1.41 at 4; occupancies 0.54 and 0.77 ms,
-// 1.18 and 0.85; FP64 displacements 14.0 and 7.6 ms at 0.6; occupancies 0.91 and 1.30 ms at 0.6, 1.71 and
-// 1.34 at 1.6.  Where the rule shares, sharing was at most 6 % slower than box by box at any overlap between
-// the measured ones.  From 48^3 cells on the line sums of one block of points exceed the L2; sharing gains
-// there too (FP32, 64^3, four displaced sites, 2.5 boxes per cell, 1600 points: 7.5 and 2.4 ms).
+// displacements 2.23 and 1.38 ms at 4 boxes per cell; occupancies 0.54 and 0.77 ms at 1.6, 1.17 and 0.85 at
+// 4; FP64 displacements 14.0 and 7.8 ms at 0.6; occupancies 0.91 and 1.30 ms at 0.6, 1.71 and 1.34 at 1.6.
+// Where the rule shares, sharing was at most 8 % slower than box by box at any overlap between the measured
+// ones, and at most 3 % in 270 random requests.  From 48^3 cells on the line sums of one block of points
+// exceed the L2; sharing gains there too (FP32, 64^3, four displaced sites, 2.5 boxes per cell, 1600 points:
+// 7.5 and 2.5 ms).
 bool cells_cheaper(bool fp64, int kind, bool diffuse, int nsite, int nsb, double cells, double norigin, double fill) {
     const int NC = kind == SB_SPIN ? 3 : 1;
     const double ns = nsite, w = nsb;
@@ -522,12 +606,13 @@ bool cells_cheaper(bool fp64, int kind, bool diffuse, int nsite, int nsb, double
     } else {
         const double pad = nsite <= 4 ? 4 : (nsite <= 8 ? 8 : 16);
         if (kind == SB_DISP) box_cell = 50 + 60 * ns, cell = 6 + 85 * ns + (wide ? 9.5 : 7.2) * w, line = 13, dw = 150 * ns;
-        else if (kind == SB_OCC) box_cell = 40 + 7 * ns, cell = 3 + 6.7 * ns + (wide ? 9.4 : 7.1) * w, line = 12;
-        else box_cell = 30 + 22 * ns, cell = wide ? 30 + 13 * pad + 33 * w : 80 + 15 * pad + 27 * w, line = 40;
+        else if (kind == SB_OCC) box_cell = 40 + 7 * ns, cell = 12 + 6.7 * ns + (wide ? 9.4 : 7.1) * w, line = 12;
+        else box_cell = 30 + 22 * ns, cell = wide ? 30 + 13 * pad + 33 * w : 100 + 15 * pad + 27 * w, line = 40;
         if (wide) line = NC;
     }
     double by_box = norigin * w * w * w * box_cell + (diffuse ? dw * cells : 0.0);
-    if (!fp64 && kind != SB_DISP) by_box *= std::pow(fill, -0.4);
+    if (!fp64 && kind != SB_DISP) by_box += 2.3 * norigin;   // per box
+    if (!fp64 && kind != SB_DISP) by_box *= std::pow(fill, -0.25);
     return cells * cell + norigin * w * w * line <= 0.95 * by_box;
 }
 
@@ -569,6 +654,9 @@ bool subbox_cells_run(ds_model *M, int kind, const SbSite *d_sites, const int4 *
     p.origins = d_org;
     p.norigin = norigin;
     for (int i = 0; i < 9; ++i) p.recip[i] = M->recip[i];
+    p.off = sizeof(T) == 4 && p.diffuse ? T(0.0625) : T(0);
+    p.off_c = (T)std::cos(TWO_PI_D * p.off);
+    p.off_s = (T)std::sin(TWO_PI_D * p.off);
     // row blocks: about eight blocks per SM
     const long long nrow = (long long)p.nmodels * p.n1 * p.n2;
     const long long want = std::max<long long>(1, 152 * 8 / blocks);
@@ -589,7 +677,7 @@ bool subbox_cells_run(ds_model *M, int kind, const SbSite *d_sites, const int4 *
         need += (count * sizeof(*ptr) + 255) & ~(size_t)255;
     };
     part(p.phi, nk * nsite);
-    part(p.e, nk * 3);
+    part(p.e, nk * 3 * (SX_RING + 1));
     part(p.Q, nk * 3);
     if (mean_b) part(p.phiB, nk * nsite);
     part(p.K, nk * NC);
@@ -597,7 +685,7 @@ bool subbox_cells_run(ds_model *M, int kind, const SbSite *d_sites, const int4 *
     if (nsb > SX_RING) part(p.A, (size_t)cells * NC * p.ld);
     if (mean_b) {
         part(p.dwp, (size_t)p.nrb * nsite * p.ld);
-        part(p.dwm, (size_t)nsite * p.ld);
+        part(p.KB, (size_t)p.ld);
     }
     part(p.partial, (size_t)nochunk * npts);
     if (ws.total + need > ctx->budget) return false;

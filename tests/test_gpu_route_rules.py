@@ -114,17 +114,21 @@ def test_subbox_points_systematic_absences_are_zero(ctx, nsb):
     assert np.all(got == 0.0)
 
 
-@pytest.mark.parametrize("prec,tag", PREC)
-def test_subbox_points_mean_term_of_an_undisplaced_crystal(ctx, prec, tag):
-    """DIFFUSE boxes of an undisplaced crystal at Bragg positions: <cos(Q.u)> = 1, the box phases are 1 and
-    2^3 cells add without rounding, so F = 8 phi and the mean term, formed in FP64 and rounded once, is
-    the same number."""
+def test_subbox_points_mean_term_of_an_undisplaced_crystal(ctx):
+    """DIFFUSE boxes of an undisplaced crystal at Bragg positions.  FP64: <cos(Q.u)> = 1, the box phases are 1
+    and 2^3 cells add without rounding, so F = 8 phi and the mean term, rounded once, is the same number.
+    FP32: the atoms' fast sine and cosine (2^-20.9 at most) and a few roundings in F and the mean leave
+    |F - K B| below 2e-6 of |F|, an intensity below 4e-12 of the Bragg peak."""
     m = _undisplaced([[0.3, 0.17, 0.71]])
+    lm = to_library(ctx, m)
     rng = np.random.default_rng(32)
     hkl = rng.integers(-6, 7, (200, 3)).astype(np.float64)
     org = syn.random_origins(rng, 1, m.cells, 360)
-    got, _ = to_library(ctx, m).subbox_points(hkl, org, disorder=2, mode=1, precision=prec, subbox_n=2)
+    got, _ = lm.subbox_points(hkl, org, disorder=2, mode=1, precision=0, subbox_n=2)
     assert np.all(got == 0.0)
+    got, _ = lm.subbox_points(hkl, org, disorder=2, mode=1, precision=1, subbox_n=2)
+    bragg, _ = lm.subbox_points(hkl, org, disorder=2, mode=0, precision=1, subbox_n=2)
+    assert np.all(got < 4e-12 * bragg)
 
 
 @pytest.mark.parametrize("prec,tag", PREC)
@@ -143,6 +147,17 @@ def test_subbox_points_shared_amplitudes_of_every_site_count(ctx, prec, tag, kin
         org = syn.random_origins(rng, 1, cells, max(2, ratio * int(np.prod(cells)) // nsb ** 3))
         got, _ = lm.subbox_points(hkl, org, disorder=code, mode=1, precision=prec, subbox_n=nsb)
         assert rel_err_of_peak(got, noise.subbox_intensity(m, kind, 1, nsb, hkl, org)) < TOL[tag]
+
+
+@pytest.mark.parametrize("prec,tag", PREC)
+def test_subbox_points_boxes_wider_than_two_rings(ctx, prec, tag):
+    """Boxes of 17 cells: three blocks of tabulated phase powers along each axis."""
+    m = syn.small_case(syn.DISP, cells=(18, 20, 18), nsite=5, nmodels=1, seed=247)
+    rng = np.random.default_rng(35)
+    hkl = rng.uniform(-1.5, 1.5, (5, 3))
+    org = syn.random_origins(rng, 1, m.cells, 40)
+    got, _ = to_library(ctx, m).subbox_points(hkl, org, disorder=2, mode=1, precision=prec, subbox_n=17)
+    assert rel_err_of_peak(got, noise.subbox_intensity(m, "disp", 1, 17, hkl, org)) < TOL[tag]
 
 
 @pytest.mark.parametrize("prec,tag", PREC)
