@@ -231,7 +231,8 @@ void launch_field_inv(const c_t<T> *in, size_t nf, T *out, const int4 *terms, in
 // The adjoint's transforms end in Re[i^n sum_k exp(ik.R) Z(k)], so only the Hermitian part of i^n Z enters.
 // With F(-G) = conj F(G) and phi(-G) = conj phi(G) it is Z with dL/dI(G) replaced by the mean of
 // dL/dI(G) and dL/dI(-G): on a grid symmetric about the origin the stored half of the k suffices, half the
-// work and memory of Z, and a half-spectrum transform (cubic FP32 supercells of 8, 16, 20 or 32 cells).
+// work of Z (its buffer is still taken for every k), and a half-spectrum transform (cubic FP32 supercells of
+// 8, 16, 20 or 32 cells).
 // fcc 32^3, 321^3 voxels, order 30: Z 9.75 -> 5.33 ms, transforms 3.33 -> 1.41 ms.
 bool adjoint_half(const Geometry &g, const int g0[3], const int cnt[3]) {
     const int n = g.n[0];
@@ -565,7 +566,7 @@ ds_status backward_run(ds_model *M, const ds_qgrid *q, const ds_opts *o, const T
     const double N = (double)nsite * g.ncell;
     const int nT = mag ? 3 : p.nT;
     const size_t nfield = (size_t)nmod * nsite * nT;
-    C *Z = (C *)ws.get(sizeof(C) * nfield * g.ncell);   // half of it when the Hermitian part is formed
+    C *Z = (C *)ws.get(sizeof(C) * nfield * g.ncell);   // the first half of it used when the Hermitian part is formed
     bool half = false;
     T *D = (T *)ws.get(sizeof(T) * nfield * g.ncell);
     const int fb = (int)std::max<size_t>(1, std::min<size_t>(nfield, (256ull << 20) / (sizeof(C) * (size_t)g.ncell)));

@@ -440,7 +440,8 @@ template <typename T> struct DwParams {
 // polynomial in the working type while x_max <= 2 (cosh x_max bounds the cancellation), else all in FP64: FP32
 // products left an error of T^2 of 1.2e-5 at x_max = 6.5 (every atom at +u or -u; 1.7e-8 in FP64).
 // 16 sites, 20^3 cells, 81^3 voxels, x_max about 0.5: the request takes 0.25 ms, 17.4 ms by the direct
-// sum (whose FP32 rotations left 1.6e-5 of the result; 1.1e-7 by the moments).  A grid of fewer voxels
+// sum (whose FP32 rotations left 1.6e-5 of the result; 1.1e-7 by the moments); x_max about 4: 4.0 ms in FP64;
+// beyond 6.6 the direct sum, 16.9 ms.  A request that takes the direct sum pays about 20 us for the decision.  A grid of fewer voxels
 // than monomials keeps the direct sum: one rotation per voxel and point costs about a monomial's product.
 constexpr int DW_PCAP = 28;
 constexpr int DW_T = (DW_PCAP + 1) * (DW_PCAP + 2) * (DW_PCAP + 3) / 6;

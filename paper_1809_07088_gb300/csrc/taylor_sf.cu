@@ -406,7 +406,8 @@ bool taylor_sf_plan(const Geometry &g, const GridMap &gm, int P, int nsite, size
         }
     }
     // register widths: odd (rows of X in distinct banks); 11 and 15 since a box of 10 or 11 zones cost 13
-    // (fcc 32^3, 321^3 voxels: the volume 7.2 -> 6.3 ms, with its gradient 23.3 -> 20.6 ms)
+    // (fcc 32^3, 321^3 voxels: the volume 7.2 -> 6.3 ms, with its gradient 23.3 -> 20.6 ms) and one of 14 or
+    // 15 zones cost 17 (fcc 16^3, |h| <= 6.5 and 7: the contraction 0.60 -> 0.38 and 0.63 -> 0.48 ms)
     const int zrs[6] = {5, 9, 11, 13, 15, 17};
     int zr = 0;
     for (int z : zrs)
